@@ -190,7 +190,7 @@ typedef struct {
   double residual_max;       /* max over substeps of the final
                                 ||M^-1/2 grad|| / max(||M^1/2 v||, ||M^-1/2 J^T gamma||) */
   int32_t status_bits;       /* OR of (1 << mpm_status) seen on the device */
-  int32_t p2g_global_chunks; /* P2G particle chunks too spread for one shared tile */
+  int32_t p2g_global_chunks; /* 0 (no P2G form has chunks too spread for a shared tile) */
   /* device time of the contact solve's phases, summed over substeps [us]:
      contact-node list, gradient/Hessian scatter (G), node solve (N),
      line-search passes, impulses */
@@ -493,8 +493,9 @@ mpm_status mpm_synchronize(mpm_ctx* ctx);
 
 /* Options. MPM_OPT_PROFILE: nonzero records CUDA events around each phase of
    each substep (read with mpm_get_phase_times). MPM_OPT_SORT_EVERY: sort the
-   particles every k-th time step (default 1). MPM_OPT_P2G_CHUNK: particles
-   per P2G thread block (256, 512 or 1024; default 256). MPM_OPT_GRAPHS:
+   particles every k-th time step (default 1). MPM_OPT_P2G_CHUNK: 256,
+   512 or 1024 (default 256); accepted, without effect: P2G's launch shape
+   follows from the particle count. MPM_OPT_GRAPHS:
    nonzero (default) records each step's launch sequence once as a CUDA graph
    and replays it while the particle count, substep count, h, solver
    parameters, body count and launch options stay the same (a change
@@ -520,12 +521,8 @@ mpm_status mpm_synchronize(mpm_ctx* ctx);
    MPM_OPT_CLUSTER_BLOCKS: thread blocks (SMs) in that cluster, a power of two
    up to the largest the device schedules (0, the default: the largest, 16 on
    GB300).
-   MPM_OPT_P2G_FORM: how a warp combines the contributions of particles that
-   share a cell: MPM_P2G_GATHER (0, the default; lane j sums node j of a
-   cell's stencil over the cell's particles, fastest at several particles per
-   cell) or MPM_P2G_SCATTER (1; each lane computes its own particle's 27
-   contributions and lanes of one cell combine them by shuffles, fastest at
-   about one particle per cell). Same results up to rounding order. */
+   MPM_OPT_P2G_FORM: MPM_P2G_GATHER (0, the default) or MPM_P2G_SCATTER (1);
+   accepted, without effect: one form of P2G serves every particle density. */
 enum {
   MPM_OPT_PROFILE = 1,
   MPM_OPT_SORT_EVERY = 2,
@@ -607,8 +604,8 @@ mpm_status mpm_batch_synchronize(mpm_batch* batch, int32_t* status, mpm_step_sta
 
 /* Launch options of the batch (autotuned by the Python binding):
    MPM_BATCH_OPT_GRAPHS: nonzero (default) replays the step as a CUDA graph;
-   MPM_BATCH_OPT_P2G_CHUNK: particles per P2G thread block, 256, 512 or 1024
-     (32, 64 or 128 per warp tile; default 256);
+   MPM_BATCH_OPT_P2G_CHUNK: 256, 512 or 1024 (default 256); accepted, without
+     effect (as MPM_OPT_P2G_CHUNK);
    MPM_BATCH_OPT_G2P_THREADS: threads (= particles) per G2P block, 64 to 512
      in multiples of 32 (default 256);
    MPM_BATCH_OPT_GRID_PARTICLES: a scene gets one grid-phase block per this

@@ -404,7 +404,7 @@ cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_s
     launch_sparse_map(ctx->g, ctx->G, ctx->P[cur], n, ctx->slot_d, ctx->status, ctx->num_sms, s);
   }
   mark_phase(ctx, MPM_PHASE_P2G);
-  launch_p2g(pa, ctx->p2g_chunk, ctx->p2g_form, s);
+  launch_p2g(pa, s);
   mark_phase(ctx, MPM_PHASE_GRID);
   launch_grid(ctx->g, ctx->G, hf, ctx->num_sms, ctx->stats, s);
   if (warm_rec >= 0 && ctx->tape_pool)
@@ -605,11 +605,13 @@ mpm_status mpm_create(const mpm_grid_spec* spec, void* cuda_stream, mpm_ctx** ou
   const int64_t cap = ctx->cap;
   const int64_t ccap = spec->max_contacts;
   bool ok = true;
+  // planes of a multiple of 32 particles: P2G copies them 16 bytes at a time
+  const int64_t pcap = (cap + 31) / 32 * 32;
   for (int s = 0; s < 2; ++s) {
-    ok = ok && dalloc(&ctx->pbuf[s], (size_t)kPlanes * cap) == cudaSuccess;
+    ok = ok && dalloc(&ctx->pbuf[s], (size_t)kPlanes * pcap) == cudaSuccess;
     ok = ok && dalloc(&ctx->pidbuf[s], cap) == cudaSuccess;
-    ok = ok && dalloc(&ctx->grpbuf[s], cap) == cudaSuccess;
-    if (ok) ctx->P[s] = make_particles(ctx->pbuf[s], ctx->pidbuf[s], ctx->grpbuf[s], cap);
+    ok = ok && dalloc(&ctx->grpbuf[s], pcap) == cudaSuccess;
+    if (ok) ctx->P[s] = make_particles(ctx->pbuf[s], ctx->pidbuf[s], ctx->grpbuf[s], pcap);
   }
   const size_t nn = ctx->n_nodes;
   ok = ok && dalloc(&ctx->G.mp, nn) == cudaSuccess && dalloc(&ctx->G.vs, nn) == cudaSuccess &&

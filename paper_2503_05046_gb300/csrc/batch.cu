@@ -31,6 +31,7 @@ struct mpm_batch {
   // launch options
   bool use_graphs = true;
   int p2g_chunk = 256;
+  long long n_all = 0;  // particles of all members, as the work lists have them
   int g2p_threads = 256;
   int grid_particles = 2048;
   int solve_blocks = 1;  // blocks (one cluster) per scene's contact solve
@@ -163,7 +164,9 @@ void build_records(mpm_batch* b, float h, const mpm_solver_params& sp) {
 std::vector<int2> build_work(mpm_batch* b) {
   std::vector<int2> w;
   const int ns = (int)b->ctx.size();
-  const int p2g_per = p2g_block_particles(b->p2g_chunk);
+  b->n_all = 0;
+  for (int s = 0; s < ns; ++s) b->n_all += b->ctx[s]->n;
+  const int p2g_per = p2g_block_particles(b->n_all);
   for (int s = 0; s < ns; ++s) {
     const int blocks = ceil_div(b->ctx[s]->n, p2g_per);
     for (int k = 0; k < blocks; ++k) w.push_back(make_int2(s, k));
@@ -190,7 +193,7 @@ cudaError_t enqueue(mpm_batch* b, int n_substeps, double dt) {
   const int ns = (int)b->ctx.size();
   launch_batch_begin(b->rig_d, ns, s);
   for (int k = 0; k < n_substeps; ++k) {
-    launch_p2g_batch(b->p2g_d, b->work_d, b->n_p2g, b->p2g_chunk, s);
+    launch_p2g_batch(b->p2g_d, b->work_d, b->n_p2g, b->n_all, s);
     launch_grid_batch(b->grid_d, b->work_d + b->n_p2g, b->n_grid, s);
     const cudaError_t e = launch_solve_batch(b->solve_d, b->order_d, ns, b->solve_blocks, s);
     if (e != cudaSuccess) return e;

@@ -73,8 +73,7 @@ struct P2GArgs {
   float* fext;  // cloth: per-particle mesh forces, 3 planes of fext_stride (null: none); P2G zeroes them
   long long fext_stride;
 };
-// form: MPM_P2G_GATHER or MPM_P2G_SCATTER
-void launch_p2g(const P2GArgs& a, int chunk, int form, cudaStream_t s);
+void launch_p2g(const P2GArgs& a, cudaStream_t s);
 cudaError_t p2g_prepare();  // once per device: the kernel's shared-memory attributes
 
 // ---- grid.cu: active-block compaction and grid update ----
@@ -268,7 +267,7 @@ void launch_g2p(const G2PArgs& a, cudaStream_t s);
 
 // ---- batched launches: one per phase over many scenes' work items ----
 // work[b] = (scene, block index within the scene); args: per scene, device
-// memory. P2G blocks hold p2g_block_particles(chunk) particles, G2P blocks
+// memory. P2G blocks hold p2g_block_particles(n) particles, n all scenes', G2P blocks
 // `threads` (<= 512); the grid phases give each scene n_slices blocks.
 struct GridBatchArgs {
   GridDev g;
@@ -277,8 +276,8 @@ struct GridBatchArgs {
   int n_slices;
   DevStats* stats;
 };
-int p2g_block_particles(int chunk);
-void launch_p2g_batch(const P2GArgs* args, const int2* work, int n_work, int chunk, cudaStream_t s);
+int p2g_block_particles(long long n);
+void launch_p2g_batch(const P2GArgs* args, const int2* work, int n_work, long long n, cudaStream_t s);
 void launch_grid_batch(const GridBatchArgs* args, const int2* work, int n_work, cudaStream_t s);
 // each scene's contact solve by one block or one cluster of 2, 4 or 8 blocks,
 // scenes in `order` (device, n_scenes entries)
