@@ -2,8 +2,8 @@
 // op (3), MLS-MPM): v_p = sum_i w v_i, C_p = (4/dx^2) sum_i w v_i (x_i - x_p)^T,
 // x_p += h v_p, F_p <- (I + h C_p) F_p, then the Drucker-Prager return map for
 // sand, fused with the stress update: the Kirchhoff stress of the new F is
-// stored for the next P2G, so one SVD per particle and substep serves both
-// the plasticity and the stress. One thread per particle; particle planes are read and written with
+// stored for the next P2G (elastic: a polynomial of F^T F - I; sand: one SVD per
+// particle and substep serves both the plasticity and the stress). One thread per particle; particle planes are read and written with
 // coalesced loads and stores, grid velocities are gathered from L2.
 //
 // Block 0 also closes the substep: it records the contact / active-block
@@ -15,7 +15,11 @@ namespace mpmcr {
 
 namespace {
 
-constexpr int kThreads = 256;
+// 128 threads, seven blocks per SM (72 registers, no spills): 1M elastic
+// particles 49.0 us per launch against 52.6 with 64 registers (four blocks of
+// 256) and 55.5 with 80 (66 us with the decomposition for every particle); the
+// bound is the 216 B per particle that the planes move, 32 us at HBM's rate.
+constexpr int kThreads = 128;
 
 // Block `block` of G2P over one scene's particles, blockDim.x particles (a
 // thread block of the single-scene launch, or a work item of the batched one).
@@ -134,7 +138,7 @@ __device__ __forceinline__ void g2p_block(const G2PArgs& a, int block) {
 
 // kDense: a dense grid's node addresses (no block-table lookup)
 template <bool kDense>
-__global__ void __launch_bounds__(kThreads, 4) k_g2p(G2PArgs a) {
+__global__ void __launch_bounds__(kThreads, 7) k_g2p(G2PArgs a) {
   g2p_block<kDense>(a, blockIdx.x);
 }
 
