@@ -183,10 +183,10 @@ SMALL_SORT_MAX = 8192  # particles the library sorts in one thread block
 def kernel_launches_per_step(res, n_substeps, n_bodies=0, n_particles=None):
     """Kernels one mpm_step launches: the sort (above 8,192 particles the
     radix sort: keys, five kernels per 8-bit digit pass, permutation; up to
-    it one sorting block and the permutation), per substep P2G, block
-    compaction, grid update, the two solve kernels (the cluster one and the
-    cooperative one, of which the contact count picks one to work) and G2P,
-    and with bodies the rigid update after the substeps."""
+    it one sorting block and the permutation), per substep P2G, grid update,
+    the three solve kernels (one block, the cluster and the cooperative one,
+    of which the contacts pick one to work) and G2P, and with bodies the rigid
+    update after the substeps."""
     if n_particles is not None and n_particles <= SMALL_SORT_MAX:
         sort = 2
     else:

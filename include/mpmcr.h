@@ -556,7 +556,7 @@ mpm_status mpm_get_phase_times(mpm_ctx* ctx, double* ms, int64_t* launches, int3
    Launch overhead dominates small scenes (Sec. V-A: the per-substep kernel
    launches and host-device synchronisations). A batch advances n
    independent contexts together so that one substep of ALL of them costs
-   five launches: P2G (with contact registration), block compaction, grid
+   five launches: P2G (with contact registration), grid
    update, contact solve (Alg. 1) and G2P, each over a work list of
    (scene, thread block) items that covers every scene, plus one launch at
    the start and one at the end of the time step (the latter moves every

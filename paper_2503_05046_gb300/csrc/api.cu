@@ -406,7 +406,7 @@ cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_s
   mark_phase(ctx, MPM_PHASE_P2G);
   launch_p2g(pa, s);
   mark_phase(ctx, MPM_PHASE_GRID);
-  launch_grid(ctx->g, ctx->G, hf, ctx->num_sms, ctx->stats, s);
+  launch_grid(ctx->g, ctx->G, hf, ctx->num_sms, s);
   if (warm_rec >= 0 && ctx->tape_pool)
     launch_tape_warm(ctx->g, ctx->G, ctx->tape_recs, warm_rec, ctx->tape_pool, ctx->num_sms, s);
   SolveArgs sa;
@@ -417,6 +417,7 @@ cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_s
   sa.wait_extra = ctx->wait_test ? 1 : 0;
   sa.poison = ctx->poison;
   sa.cluster_max = cluster_contacts(ctx);
+  sa.small_max = 0;  // (set by the launch)
   mark_phase(ctx, MPM_PHASE_SOLVE);
   const cudaError_t e = launch_solve(sa, solve_blocks, ctx->cluster_blocks, s);
   if (e != cudaSuccess) return e;
@@ -1693,7 +1694,7 @@ mpm_status mpm_backward(mpm_ctx* ctx, int32_t mem_kind, const float* x_bar, cons
       CU(launch_adjoint(a, ctx->adj_blocks, s));
       launch_grid_adjoint(ba, ctx->num_sms, s);
       launch_p2g_adjoint(ba, s);
-      launch_reset_counters(ctx->G, ctx->C, ctx->bar, s);
+      launch_reset_counters(ctx->G, ctx->C, ctx->bar, ctx->stats, s);
       CU(cudaGetLastError());
       in = 1 - in;
       ++substeps;

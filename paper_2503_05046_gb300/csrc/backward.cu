@@ -616,7 +616,8 @@ __global__ void __launch_bounds__(kThreads) k_p2g_adjoint(BackwardArgs a) {
 
 // The per-substep counters that G2P resets in the forward pass (the
 // backward replays P2G, grid and solve without G2P).
-__global__ void k_reset_counters(GridArrays G, Contacts C, unsigned* bar) {
+__global__ void k_reset_counters(GridArrays G, Contacts C, unsigned* bar, DevStats* stats) {
+  stats->last_active = *G.n_act;
   *C.count = 0;
   *G.n_act = 0;
   *G.n_cnodes = 0;
@@ -728,8 +729,9 @@ void launch_p2g_adjoint(const BackwardArgs& a, cudaStream_t s) {
   if (a.n > 0) k_p2g_adjoint<<<(a.n + kThreads - 1) / kThreads, kThreads, 0, s>>>(a);
 }
 
-void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, cudaStream_t s) {
-  k_reset_counters<<<1, 1, 0, s>>>(G, C, bar);
+void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, DevStats* stats,
+                           cudaStream_t s) {
+  k_reset_counters<<<1, 1, 0, s>>>(G, C, bar, stats);
 }
 
 void launch_tape_save(const GridDev& g, const GridArrays& G, int* counters, int2* recs, int rec_cap, float4* pool,

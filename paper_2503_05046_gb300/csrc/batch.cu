@@ -144,6 +144,7 @@ void build_records(mpm_batch* b, float h, const mpm_solver_params& sp) {
     sa.wait_extra = 0;
     sa.poison = c->poison;
     sa.cluster_max = 0;  // one block per scene, no cluster
+    sa.small_max = 0;    // (the launches set both)
     G2PArgs& qa = b->g2p_h[s];
     qa = G2PArgs{};
     qa.g = c->g; qa.P = c->P[c->cur]; qa.n = (int)c->n; qa.groups = c->groups_d; qa.G = c->G;

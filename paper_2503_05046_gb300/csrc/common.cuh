@@ -894,24 +894,27 @@ __device__ __forceinline__ void contact_line(float phi0, float n0, float mu, flo
   L.et2 = L.et[0] * L.et[0] + L.et[1] * L.et[1] + L.et[2] * L.et[2];
 }
 
-// d/dalpha and d2/dalpha2 of l_c(v_c + alpha e)
-__device__ __forceinline__ void contact_line_eval(const ContactLine& L, float al, float& d1,
-                                                  float& d2) {
-  const float vn = fmaf(al, L.en, L.vn0);
-  float dN = 0.0f, d2N = 0.0f;
-  if (vn < L.vhat) {
-    const float a = L.phi0 - L.h * vn, c = 1.0f - L.d * vn;
-    dN = -L.hk * a * c;
-    d2N = L.hk * (L.h * c + L.d * a);
-  }
-  const float u0 = fmaf(al, L.et[0], L.vt[0]), u1 = fmaf(al, L.et[1], L.vt[1]),
-              u2 = fmaf(al, L.et[2], L.vt[2]);
-  const float s2 = u0 * u0 + u1 * u1 + u2 * u2 + L.eps2;
-  const float inv_s = rsqrtf(s2);
-  const float cs = L.mun0 * inv_s;
-  const float ute = u0 * L.et[0] + u1 * L.et[1] + u2 * L.et[2];
-  d1 = dN * L.en + cs * ute;
-  d2 = d2N * L.en * L.en + cs * (L.et2 - ute * ute * inv_s * inv_s);
+// d/dalpha and d2/dalpha2 of l_c(v_c + alpha e) at two points (paired FP32
+// operations: the line search evaluates eight per contact and pass)
+__device__ __forceinline__ void contact_line_eval2(const ContactLine& L, float2 al, float2& d1,
+                                                   float2& d2) {
+  auto dup = [](float x) { return make_float2(x, x); };
+  const float2 vn = __ffma2_rn(al, dup(L.en), dup(L.vn0));
+  const float2 a = __ffma2_rn(dup(-L.h), vn, dup(L.phi0)), c = __ffma2_rn(dup(-L.d), vn, dup(1.0f));
+  float2 dN = __fmul2_rn(__fmul2_rn(dup(-L.hk), a), c);
+  float2 d2N = __fmul2_rn(dup(L.hk), __ffma2_rn(dup(L.h), c, __fmul2_rn(dup(L.d), a)));
+  if (!(vn.x < L.vhat)) dN.x = d2N.x = 0.0f;
+  if (!(vn.y < L.vhat)) dN.y = d2N.y = 0.0f;
+  const float2 u0 = __ffma2_rn(al, dup(L.et[0]), dup(L.vt[0])), u1 = __ffma2_rn(al, dup(L.et[1]), dup(L.vt[1])),
+               u2 = __ffma2_rn(al, dup(L.et[2]), dup(L.vt[2]));
+  const float2 s2 = __ffma2_rn(u0, u0, __ffma2_rn(u1, u1, __ffma2_rn(u2, u2, dup(L.eps2))));
+  const float2 inv_s = make_float2(rsqrtf(s2.x), rsqrtf(s2.y));
+  const float2 cs = __fmul2_rn(dup(L.mun0), inv_s);
+  const float2 ute = __ffma2_rn(u0, dup(L.et[0]), __ffma2_rn(u1, dup(L.et[1]), __fmul2_rn(u2, dup(L.et[2]))));
+  d1 = __ffma2_rn(dN, dup(L.en), __fmul2_rn(cs, ute));
+  const float2 q = __fmul2_rn(ute, inv_s);
+  const float2 t = __ffma2_rn(make_float2(-q.x, -q.y), q, dup(L.et2));
+  d2 = __ffma2_rn(d2N, dup(L.en * L.en), __fmul2_rn(cs, t));
 }
 
 // A batched launch's per-scene argument record, copied from global into

@@ -34,6 +34,9 @@ __device__ __forceinline__ void g2p_block(const G2PArgs& a, int block) {
       atomicMax(&a.stats->contacts_max, nc);
       atomicAdd(&a.stats->contacts_total, (unsigned long long)nc);
       atomicAdd(&a.stats->substeps, 1);
+      const int n_act = *a.G.n_act;
+      atomicMax(&a.stats->active_blocks_max, n_act);
+      a.stats->last_active = n_act;
       *a.C.count = 0;
       *a.G.n_act = 0;
       *a.G.n_cnodes = 0;

@@ -1,4 +1,4 @@
-// grid.cu -- active-block compaction and the grid update of the free-motion
+// grid.cu -- the active-block list and the grid update of the free-motion
 // solve (Sec. V-A op (2): v* = p / m + h g on every node with mass), with the
 // domain walls held at zero velocity.
 //
@@ -75,49 +75,36 @@ __global__ void k_compact_sparse(uint8_t* __restrict__ mark, int n_blocks, int* 
                 act, n_act, slot_tab, pool, status);
 }
 
-__global__ void k_compact(uint8_t* __restrict__ mark, int n_blocks, int* __restrict__ act,
-                          int* __restrict__ n_act) {
-  compact_range(mark, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, n_blocks,
-                act, n_act);
+// The grid update of one node: cell `cell` of grid block `blk`, stored at
+// `node`. Returns m |v*|^2 of a free node.
+__device__ __forceinline__ float update_node(const GridDev& g, const GridArrays& G, float h, int blk,
+                                             int cell, int node) {
+  const float4 mp = G.mp[node];
+  float4 vs = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int bx = blk % g.nbx, by = (blk / g.nbx) % g.nby, bz = blk / (g.nbx * g.nby);
+  const int i = bx * 4 + (cell & 3), j = by * 4 + ((cell >> 2) & 3), k = bz * 4 + (cell >> 4);
+  const bool wall = i < g.bc || j < g.bc || k < g.bc || i >= g.rx - g.bc || j >= g.ry - g.bc ||
+                    k >= g.rz - g.bc;
+  float p2 = 0.f;
+  if (mp.x > 0.0f) {
+    const float inv_m = 1.0f / mp.x;
+    vs.x = wall ? 0.0f : mp.y * inv_m + h * g.gx;
+    vs.y = wall ? 0.0f : mp.z * inv_m + h * g.gy;
+    vs.z = wall ? 0.0f : mp.w * inv_m + h * g.gz;
+    vs.w = mp.x;
+    if (!wall) p2 = mp.x * (vs.x * vs.x + vs.y * vs.y + vs.z * vs.z);
+  }
+  G.mp[node] = make_float4(0.f, 0.f, 0.f, 0.f);
+  G.vs[node] = vs;
+  // .w flags a Dirichlet node for the contact solve
+  G.v[node] = make_float4(vs.x, vs.y, vs.z, wall ? 1.f : 0.f);
+  G.vlo[node] = make_float4(0.f, 0.f, 0.f, 0.f);
+  return p2;
 }
 
-// The grid update of nodes t = start, start + stride, ... of the active
-// blocks' nodes; `first`: the thread that records the active-block count.
-__device__ __forceinline__ void grid_update_range(const GridDev& g, const GridArrays& G, float h,
-                                                  DevStats* stats, long long start,
-                                                  long long stride, bool first) {
-  const int n_act = *G.n_act;
-  if (first) {
-    atomicMax(&stats->active_blocks_max, n_act);
-    stats->last_active = n_act;
-    if (g.slot) *G.n_mapped = n_act;  // the list the slot table now holds
-  }
-  const long long total = (long long)active_with_storage(g, n_act) * kBlockNodes;
-  float p2 = 0.f;  // sum of m |v*|^2 over free nodes (the momentum norm of Alg. 1)
-  for (long long t = start; t < total; t += stride) {
-    const int blk = G.act[t >> 6];
-    const int cell = (int)(t & 63);
-    const int node = active_storage_block(g, G.act, (int)(t >> 6)) * kBlockNodes + cell;
-    const float4 mp = G.mp[node];
-    float4 vs = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int bx = blk % g.nbx, by = (blk / g.nbx) % g.nby, bz = blk / (g.nbx * g.nby);
-    const int i = bx * 4 + (cell & 3), j = by * 4 + ((cell >> 2) & 3), k = bz * 4 + (cell >> 4);
-    const bool wall = i < g.bc || j < g.bc || k < g.bc || i >= g.rx - g.bc ||
-                      j >= g.ry - g.bc || k >= g.rz - g.bc;
-    if (mp.x > 0.0f) {
-      const float inv_m = 1.0f / mp.x;
-      vs.x = wall ? 0.0f : mp.y * inv_m + h * g.gx;
-      vs.y = wall ? 0.0f : mp.z * inv_m + h * g.gy;
-      vs.z = wall ? 0.0f : mp.w * inv_m + h * g.gz;
-      vs.w = mp.x;
-      if (!wall) p2 += mp.x * (vs.x * vs.x + vs.y * vs.y + vs.z * vs.z);
-    }
-    G.mp[node] = make_float4(0.f, 0.f, 0.f, 0.f);
-    G.vs[node] = vs;
-    // .w flags a Dirichlet node for the contact solve
-    G.v[node] = make_float4(vs.x, vs.y, vs.z, wall ? 1.f : 0.f);
-    G.vlo[node] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+// Adds the threads' sums of m |v*|^2 over free nodes (the momentum norm of
+// Alg. 1) to the substep's.
+__device__ __forceinline__ void add_momentum_norm(const GridArrays& G, float p2) {
   __shared__ double s_p2[32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) p2 += __shfl_xor_sync(0xffffffffu, p2, o);
@@ -130,43 +117,87 @@ __device__ __forceinline__ void grid_update_range(const GridDev& g, const GridAr
   }
 }
 
-__global__ void __launch_bounds__(256) k_grid_update(GridDev g, GridArrays G, float h,
-                                                     DevStats* stats) {
-  grid_update_range(g, G, h, stats, (long long)blockIdx.x * blockDim.x + threadIdx.x,
+// The grid update of a dense grid straight from P2G's marks: warp `first` of
+// `n_warps` takes blocks first, first + n_warps, ..., 32 marks at a time (so
+// that neighbouring blocks, which are active together, go to different warps),
+// appends its marked blocks to the active list and updates their 64 nodes. One
+// launch instead of a compaction and an update; G2P closes the substep's count.
+__device__ __forceinline__ void grid_dense_range(const GridDev& g, const GridArrays& G, float h,
+                                                 int first, int n_warps) {
+  const int lane = threadIdx.x & 31;
+  const int n_blocks = g.nbx * g.nby * g.nbz;
+  float p2 = 0.f;
+  for (int base = first; base < n_blocks; base += 32 * n_warps) {
+    const int b = base + lane * n_warps;
+    const bool on = b < n_blocks && G.mark[b] != 0;
+    unsigned left = __ballot_sync(0xffffffffu, on);
+    if (left == 0u) continue;
+    int slot0 = 0;
+    if (lane == 0) slot0 = atomicAdd(G.n_act, __popc(left));
+    slot0 = __shfl_sync(0xffffffffu, slot0, 0);
+    if (on) {
+      G.act[slot0 + __popc(left & ((1u << lane) - 1u))] = b;
+      G.mark[b] = 0;
+    }
+    for (; left; left &= left - 1u) {
+      const int blk = base + (__ffs(left) - 1) * n_warps;
+      p2 += update_node(g, G, h, blk, lane, blk * kBlockNodes + lane);
+      p2 += update_node(g, G, h, blk, 32 + lane, blk * kBlockNodes + 32 + lane);
+    }
+  }
+  add_momentum_norm(G, p2);
+}
+
+__global__ void __launch_bounds__(256) k_grid_update_dense(GridDev g, GridArrays G, float h) {
+  grid_dense_range(g, G, h, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5),
+                   (int)(gridDim.x * (blockDim.x >> 5)));
+}
+
+// The grid update of nodes t = start, start + stride, ... of the active
+// blocks' nodes; `first`: the thread that notes the mapped list's length.
+__device__ __forceinline__ void grid_update_range(const GridDev& g, const GridArrays& G, float h,
+                                                  long long start, long long stride, bool first) {
+  const int n_act = *G.n_act;
+  if (first && g.slot) *G.n_mapped = n_act;  // the list the slot table now holds
+  const long long total = (long long)active_with_storage(g, n_act) * kBlockNodes;
+  float p2 = 0.f;
+  for (long long t = start; t < total; t += stride) {
+    const int cell = (int)(t & 63);
+    p2 += update_node(g, G, h, G.act[t >> 6], cell,
+                      active_storage_block(g, G.act, (int)(t >> 6)) * kBlockNodes + cell);
+  }
+  add_momentum_norm(G, p2);
+}
+
+__global__ void __launch_bounds__(256) k_grid_update(GridDev g, GridArrays G, float h) {
+  grid_update_range(g, G, h, (long long)blockIdx.x * blockDim.x + threadIdx.x,
                     (long long)gridDim.x * blockDim.x, blockIdx.x == 0 && threadIdx.x == 0);
 }
 
 // Batched: thread block b is slice work[b].y of work[b].x's scene; a scene's
-// n_slices blocks stride together over its marks (compaction) or its active
-// nodes (update)
-__global__ void __launch_bounds__(256) k_compact_batch(const GridBatchArgs* __restrict__ args,
-                                                       const int2* __restrict__ work) {
-  const int2 wk = work[blockIdx.x];
-  const GridBatchArgs& a = args[wk.x];
-  compact_range(a.G.mark, wk.y * blockDim.x + threadIdx.x, a.n_slices * blockDim.x,
-                a.g.nbx * a.g.nby * a.g.nbz, a.G.act, a.G.n_act);
-}
-
+// n_slices blocks go over its marks together
 __global__ void __launch_bounds__(256) k_grid_update_batch(const GridBatchArgs* __restrict__ args,
                                                            const int2* __restrict__ work) {
   __shared__ GridBatchArgs s_a;
   const int2 wk = work[blockIdx.x];
   load_args(args + wk.x, s_a);
   __syncthreads();
-  grid_update_range(s_a.g, s_a.G, s_a.h, s_a.stats, (long long)wk.y * blockDim.x + threadIdx.x,
-                    (long long)s_a.n_slices * blockDim.x, wk.y == 0 && threadIdx.x == 0);
+  const int warps = blockDim.x >> 5;
+  grid_dense_range(s_a.g, s_a.G, s_a.h, wk.y * warps + (int)(threadIdx.x >> 5), s_a.n_slices * warps);
 }
 
 }  // namespace
 
-void launch_grid(const GridDev& g, const GridArrays& G, float h, int num_sms, DevStats* stats,
-                 cudaStream_t s) {
-  int n_blocks = g.nbx * g.nby * g.nbz;
-  int cb = (n_blocks + 255) / 256;
-  cb = cb > num_sms * 8 ? num_sms * 8 : cb;
-  // (a sparse grid compacted its marks before P2G)
-  if (!g.slot) k_compact<<<cb, 256, 0, s>>>(G.mark, n_blocks, G.act, G.n_act);
-  k_grid_update<<<num_sms * 8, 256, 0, s>>>(g, G, h, stats);
+void launch_grid(const GridDev& g, const GridArrays& G, float h, int num_sms, cudaStream_t s) {
+  const int n_blocks = g.nbx * g.nby * g.nbz;
+  if (g.slot) {  // (compacted before P2G)
+    k_grid_update<<<num_sms * 8, 256, 0, s>>>(g, G, h);
+    return;
+  }
+  // a warp per two blocks of the domain, up to eight thread blocks per SM
+  int tb = (n_blocks + 15) / 16;
+  tb = tb > num_sms * 8 ? num_sms * 8 : tb;
+  k_grid_update_dense<<<tb, 256, 0, s>>>(g, G, h);
 }
 
 void launch_sparse_map(const GridDev& g, const GridArrays& G, const Particles& P, int n,
@@ -183,7 +214,6 @@ void launch_sparse_map(const GridDev& g, const GridArrays& G, const Particles& P
 
 void launch_grid_batch(const GridBatchArgs* args, const int2* work, int n_work, cudaStream_t s) {
   if (n_work <= 0) return;
-  k_compact_batch<<<n_work, 256, 0, s>>>(args, work);
   k_grid_update_batch<<<n_work, 256, 0, s>>>(args, work);
 }
 

@@ -77,8 +77,7 @@ void launch_p2g(const P2GArgs& a, cudaStream_t s);
 cudaError_t p2g_prepare();  // once per device: the kernel's shared-memory attributes
 
 // ---- grid.cu: active-block compaction and grid update ----
-void launch_grid(const GridDev& g, const GridArrays& G, float h, int num_sms, DevStats* stats,
-                 cudaStream_t s);
+void launch_grid(const GridDev& g, const GridArrays& G, float h, int num_sms, cudaStream_t s);
 // block-sparse grids, before P2G: the substep's blocks marked from the
 // particles' stencils, compacted and given storage (slot_tab = g.slot)
 void launch_sparse_map(const GridDev& g, const GridArrays& G, const Particles& P, int n,
@@ -105,9 +104,10 @@ struct SolveArgs {
   int wait_extra;     // 0; 1 makes every grid barrier wait for one block too many (test)
   int* poison;        // nonzero after a barrier gave up (set and cleared by the solve)
   int cluster_max;    // up to this many contacts one thread-block cluster solves (0: never)
+  int small_max;      // up to this many the one-block kernel may have solved (set by the launchers)
 };
-// the cluster kernel (cluster_blocks > 0 and a.cluster_max > 0), then the
-// cooperative one; each returns at once when the contact count is the other's
+// the one-block and the cluster kernel (cluster_blocks > 0 and a.cluster_max > 0),
+// then the cooperative one; each returns at once when the contacts are another's
 cudaError_t launch_solve(const SolveArgs& a, int grid_blocks, int cluster_blocks, cudaStream_t s);
 int solve_cluster_blocks();  // largest cluster (16, 8 or 4 blocks) the device holds; 0: none
 int solve_block_size();
@@ -182,7 +182,8 @@ struct BackwardArgs {
 void launch_g2p_adjoint(const BackwardArgs& a, cudaStream_t s);
 void launch_grid_adjoint(const BackwardArgs& a, int num_sms, cudaStream_t s);
 void launch_p2g_adjoint(const BackwardArgs& a, cudaStream_t s);
-void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, cudaStream_t s);
+void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, DevStats* stats,
+                           cudaStream_t s);
 void launch_slot_map(const Particles& P, int n, int* slot_of, cudaStream_t s);
 // taped solutions: append the contact-node velocities after a solve (counters:
 // [0] pool fill, [1] records written); scatter record r over v*

@@ -65,6 +65,27 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
   return v;
 }
 
+// Phase times of a solve by the SM's clock, scaled to nanoseconds at the end by
+// the global timer (which takes far longer to read than a phase boundary may).
+struct PhaseClock {
+  unsigned long long t[5], first, mark, ns0;
+  __device__ __forceinline__ void start() {
+    t[0] = t[1] = t[2] = t[3] = t[4] = 0ull;
+    ns0 = global_ns();
+    first = mark = (unsigned long long)clock64();
+  }
+  __device__ __forceinline__ void lap(int ph) {
+    const unsigned long long now = (unsigned long long)clock64();
+    t[ph] += now - mark;
+    mark = now;
+  }
+  __device__ __forceinline__ void finish() {  // t in nanoseconds
+    const float scale = (float)(global_ns() - ns0) / fmaxf((float)(mark - first), 1.f);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) t[k] = (unsigned long long)((float)t[k] * scale);
+  }
+};
+
 struct Barrier {
   unsigned* bar;  // arrival counters (kBarWords, zeroed between launches)
   unsigned n;     // the participating blocks
@@ -151,6 +172,27 @@ __device__ __forceinline__ void df_acc(float& S, float& E, float2 x) {
   E += e + x.y;
 }
 
+// Warp sums of 16 values by a reduce-scatter butterfly: after the exchange
+// over lane bit b each lane keeps half of its values (those whose index bit b
+// equals its lane bit b), so lane l ends with value l & 15 summed over the warp
+// (16 shuffles instead of 80).
+__device__ __forceinline__ float warp_sums16(const float (&v)[16], int lane) {
+  float x[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) x[i] = v[i];
+#pragma unroll
+  for (int b = 0, m = 8; b < 4; ++b, m >>= 1) {
+    const bool hi = (lane >> b) & 1;
+#pragma unroll
+    for (int j = 0; j < m; ++j) {
+      const float keep = hi ? x[2 * j + 1] : x[2 * j];
+      const float send = hi ? x[2 * j] : x[2 * j + 1];
+      x[j] = keep + __shfl_xor_sync(0xffffffffu, send, 1 << b);
+    }
+  }
+  return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 16);
+}
+
 // Block sums of NV per-thread values, exchanged through per-block slots and
 // summed by every block in the same fixed order (deterministic). Returns the
 // double-float totals in s_tot (shared) and false if the barrier expired.
@@ -163,24 +205,7 @@ __device__ bool reduce_all(const float (&v)[NV], float2* part, Barrier& B, float
   static_assert(NV <= kWarps && NV <= kRedWidth, "one warp per reduced value");
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if constexpr (NV == 16) {
-    // reduce-scatter butterfly: after the exchange over lane bit b each lane
-    // keeps half of its values (those whose index bit b equals its lane bit
-    // b), so lane l ends with value l & 15 summed over the warp (16 shuffles
-    // instead of 80)
-    float x[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) x[i] = v[i];
-#pragma unroll
-    for (int b = 0, m = 8; b < 4; ++b, m >>= 1) {
-      const bool hi = (lane >> b) & 1;
-#pragma unroll
-      for (int j = 0; j < m; ++j) {
-        const float keep = hi ? x[2 * j + 1] : x[2 * j];
-        const float send = hi ? x[2 * j] : x[2 * j + 1];
-        x[j] = keep + __shfl_xor_sync(0xffffffffu, send, 1 << b);
-      }
-    }
-    const float t = x[0] + __shfl_xor_sync(0xffffffffu, x[0], 16);
+    const float t = warp_sums16(v, lane);
     if (lane < 16) s_red[w][lane] = t;
   } else {
 #pragma unroll
@@ -379,17 +404,18 @@ struct LineSearch {
     pt = k == 0 ? 0.f : exp2f(2.0f * (float)(k - 6));
   }
   // f' = B + alpha A + S is formed in double-float (its terms can cancel);
-  // the bracket logic runs in FP32 (alpha is applied in FP32 anyway)
-  __device__ int update(const float2* tot, float2 A, float2 B, float rel_tol, bool last) {
+  // the bracket logic runs in FP32 (alpha is applied in FP32 anyway). tk, tk2:
+  // the contact sums of f' and f'' at this lane's point
+  __device__ int update(float2 tk, float2 tk2, float2 A, float2 B, float rel_tol, bool last) {
     const int k = threadIdx.x & (kLsPoints - 1);
     const float x = pt;
     CompSum c;
     c.S = B.x;
-    c.E = B.y + x * A.y + tot[k].y;
+    c.E = B.y + x * A.y + tk.y;
     c.add_prod(x, A.x);
-    c.add(tot[k].x);
+    c.add(tk.x);
     const float d = c.value();
-    const float d2 = (A.x + tot[kLsPoints + k].x) + (A.y + tot[kLsPoints + k].y);
+    const float d2 = (A.x + tk2.x) + (A.y + tk2.y);
     if (!have_f0) {  // the first pass's point 0 is alpha = 0
       f0 = __shfl_sync(0xffffffffu, d, 0);
       flo = f0;
@@ -400,32 +426,24 @@ struct LineSearch {
     }
     // candidates of this pass: the largest point with f' < 0 (ties: the later
     // point), the smallest with f' >= 0 (ties: the earlier), the smallest
-    // |f'| (ties: the earlier)
-    float clo = d < 0.f ? x : -1.f, cflo = d;
-    int klo = k;
-    float chi = d < 0.f ? INFINITY : x, cfhi = d;
-    int khi = k;
-    float cb = fabsf(d), cbx = x, cbd = d, cbd2 = d2;
-    int kb = k;
-#pragma unroll
-    for (int o = 1; o < kLsPoints; o <<= 1) {
-      const float olo = __shfl_xor_sync(0xffffffffu, clo, o);
-      const float oflo = __shfl_xor_sync(0xffffffffu, cflo, o);
-      const int oklo = __shfl_xor_sync(0xffffffffu, klo, o);
-      if (olo > clo || (olo == clo && oklo > klo)) { clo = olo; cflo = oflo; klo = oklo; }
-      const float ohi = __shfl_xor_sync(0xffffffffu, chi, o);
-      const float ofhi = __shfl_xor_sync(0xffffffffu, cfhi, o);
-      const int okhi = __shfl_xor_sync(0xffffffffu, khi, o);
-      if (ohi < chi || (ohi == chi && okhi < khi)) { chi = ohi; cfhi = ofhi; khi = okhi; }
-      const float ob = __shfl_xor_sync(0xffffffffu, cb, o);
-      const float obx = __shfl_xor_sync(0xffffffffu, cbx, o);
-      const float obd = __shfl_xor_sync(0xffffffffu, cbd, o);
-      const float obd2 = __shfl_xor_sync(0xffffffffu, cbd2, o);
-      const int okb = __shfl_xor_sync(0xffffffffu, kb, o);
-      if (ob < cb || (ob == cb && okb < kb)) { cb = ob; cbx = obx; cbd = obd; cbd2 = obd2; kb = okb; }
-    }
-    if (clo >= lo) { lo = clo; flo = cflo; }
-    if (chi != INFINITY && (hi < 0.f || chi < hi)) { hi = chi; fhi = cfhi; }
+    // |f'| (ties: the earlier). Points and |f'| are not negative, so their bit
+    // patterns compare as they do.
+    const bool neg = d < 0.f;
+    const int xb = __float_as_int(x);
+    const int blo = __reduce_max_sync(0xffffffffu, neg ? xb : -1);
+    const int bhi = __reduce_min_sync(0xffffffffu, neg ? 0x7f800000 : xb);
+    const int ab = __float_as_int(fabsf(d));
+    const int bb = __reduce_min_sync(0xffffffffu, ab);
+    const unsigned is_lo = __ballot_sync(0xffffffffu, neg && xb == blo) & 0xffu;
+    const unsigned is_hi = __ballot_sync(0xffffffffu, !neg && xb == bhi) & 0xffu;
+    const int kb = __ffs(__ballot_sync(0xffffffffu, ab == bb) & 0xffu) - 1;
+    const float clo = __int_as_float(blo), chi = __int_as_float(bhi), cb = __int_as_float(bb);
+    const float cflo = __shfl_sync(0xffffffffu, d, is_lo ? 31 - __clz(is_lo) : 0);
+    const float cfhi = __shfl_sync(0xffffffffu, d, is_hi ? __ffs(is_hi) - 1 : 0);
+    const float cbx = __shfl_sync(0xffffffffu, x, kb), cbd = __shfl_sync(0xffffffffu, d, kb),
+                cbd2 = __shfl_sync(0xffffffffu, d2, kb);
+    if (is_lo && clo >= lo) { lo = clo; flo = cflo; }
+    if (is_hi && chi != INFINITY && (hi < 0.f || chi < hi)) { hi = chi; fhi = cfhi; }
     if (cb < fabsf(fbest)) { best = cbx; fbest = cbd; f2best = cbd2; }
     if (!(f0 < 0.f)) { best = 0.f; return kDone; }  // no descent left at working precision
     if (fabsf(fbest) <= rel_tol * fabsf(f0) || last) return kDone;
@@ -467,6 +485,634 @@ struct LineSearch {
   }
 };
 
+// One contact node of phase N: gradient g = M (v - v*) + c, H = M + contact
+// blocks, dv = -H^-1 g (Cholesky), and the node's terms of the five grid sums
+// (G2, P2 - P*2, J2, A, B). r = v - v*.
+__device__ __forceinline__ void node_step(float m, const float4& vs, float r0, float r1, float r2,
+                                          const float4& c0, const float4& c1, float c2, float& dx,
+                                          float& dy, float& dz, float* acc) {
+  const float g0 = m * r0 + c0.x, g1 = m * r1 + c0.y, g2 = m * r2 + c0.z;
+  const float inv_m = 1.0f / m;
+  acc[0] += (g0 * g0 + g1 * g1 + g2 * g2) * inv_m;
+  // m (|v|^2 - |v*|^2) = m r . (2 v* + r)
+  acc[1] += m * (r0 * (2.f * vs.x + r0) + r1 * (2.f * vs.y + r1) + r2 * (2.f * vs.z + r2));
+  acc[2] += (c0.x * c0.x + c0.y * c0.y + c0.z * c0.z) * inv_m;
+  // H = m I + contact block; dv = -H^-1 g (Cholesky)
+  const float h00 = m + c0.w, h11 = m + c1.x, h22 = m + c1.y;
+  const float h01 = c1.z, h02 = c1.w, h12 = c2;
+  const float l00 = sqrtf(h00);
+  const float l10 = h01 / l00, l20 = h02 / l00;
+  const float l11 = sqrtf(fmaxf(h11 - l10 * l10, 1e-30f));
+  const float l21 = (h12 - l20 * l10) / l11;
+  const float l22 = sqrtf(fmaxf(h22 - l20 * l20 - l21 * l21, 1e-30f));
+  const float y0 = -g0 / l00;
+  const float y1 = (-g1 - l10 * y0) / l11;
+  const float y2 = (-g2 - l20 * y0 - l21 * y1) / l22;
+  dz = y2 / l22;
+  dy = (y1 - l21 * dz) / l11;
+  dx = (y0 - l10 * dy - l20 * dz) / l00;
+  acc[3] += m * (dx * dx + dy * dy + dz * dz);
+  acc[4] += m * (dx * r0 + dy * r1 + dz * r2);
+}
+
+// The stopping test of Alg. 1 on the grid sums, by one thread (FP64 is a
+// narrow pipe on GB300): nonzero ends the iteration. `report`: this block
+// records failures.
+__device__ __forceinline__ int stop_test(const SolveArgs& a, const float2* tot, float pstar2_hi,
+                                         float pstar2_lo, float eps_a, float eps_r, int it,
+                                         bool report, float& resid) {
+  const float2 A = tot[3], Bs = tot[4];
+  const float G2 = tot[0].x + tot[0].y, J2 = tot[2].x + tot[2].y;
+  const float P2 = (pstar2_hi + tot[1].x) + (pstar2_lo + tot[1].y);
+  const float Gn = sqrtf(G2), Pn = sqrtf(fmaxf(P2, 0.f)), Jn = sqrtf(J2);
+  const float mx = fmaxf(Pn, Jn);
+  resid = mx > 0.f ? Gn / mx : 0.f;
+  if (!(G2 == G2) || !(A.x == A.x) || !(Bs.x == Bs.x)) {
+    if (report) atomicOr(a.status, kStNan);
+    return 1;
+  }
+  if (Gn < eps_a + eps_r * mx || G2 == 0.f) return 1;  // converged
+  if (it >= a.max_iters) {
+    if (report) atomicOr(a.status, kStNotConverged);
+    return 1;
+  }
+  return 0;
+}
+
+// Impulse of contact p (valid lanes) at its velocity u: gamma = -dl_c/dv_c on
+// the particle; the body receives -gamma and its moment about the body origin
+// (Eq. (3)); the warp sums its contacts body by body into the block's sums.
+__device__ __forceinline__ void contact_impulses(const SolveArgs& a, const DevBody* s_body, int p,
+                                                 bool valid, const float4& xp, const float (&n)[3],
+                                                 float n0, int body, const float (&u)[3], int lane,
+                                                 float (*s_imp)[6]) {
+  int b = -1;
+  float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (valid) {
+    b = body;
+    const DevBody& bd = s_body[b];
+    ContactLaw L;
+    contact_law(xp.w, n0, bd.mu, bd.k, bd.d, a.h, a.eps_s, n, u, L);
+    float gr[3];
+    contact_grad(L, n, gr);
+    a.C.gamma[p] = make_float4(-gr[0], -gr[1], -gr[2], 0.f);
+    const float r0 = xp.x - bd.p[0], r1 = xp.y - bd.p[1], r2 = xp.z - bd.p[2];
+    q[0] = gr[0]; q[1] = gr[1]; q[2] = gr[2];
+    q[3] = r1 * gr[2] - r2 * gr[1];
+    q[4] = r2 * gr[0] - r0 * gr[2];
+    q[5] = r0 * gr[1] - r1 * gr[0];
+  }
+  unsigned left = __ballot_sync(0xffffffffu, b >= 0);
+  while (left) {  // one body of the warp at a time (mostly a single one)
+    const int bb = __shfl_sync(0xffffffffu, b, __ffs(left) - 1);
+    const bool mine = b == bb;
+    float t[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      t[c] = mine ? q[c] : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t[c] += __shfl_xor_sync(0xffffffffu, t[c], o);
+    }
+    if (lane == 0) {
+#pragma unroll
+      for (int c = 0; c < 6; ++c) atomicAdd(&s_imp[bb][c], t[c]);
+    }
+    left &= ~__ballot_sync(0xffffffffu, mine);
+  }
+}
+
+// one thread's record of a finished solve
+__device__ __forceinline__ void solve_stats(const SolveArgs& a, const unsigned long long (&tph)[5],
+                                            int it, int ls_passes, bool split, bool cluster, int ncn,
+                                            float resid) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) atomicAdd(&a.stats->solve_ns[k], tph[k]);
+  atomicAdd(&a.stats->iters_total, it);
+  atomicMax(&a.stats->iters_max, it);
+  atomicAdd(&a.stats->ls_evals_total, ls_passes);
+  if (split) atomicAdd(&a.stats->ls_split, 1);
+  if (cluster) atomicAdd(&a.stats->cluster, 1);
+  atomicMax(&a.stats->cnodes_max, ncn);
+  atomicMax(reinterpret_cast<int*>(&a.stats->residual_max), __float_as_int(resid));
+}
+
+// ---- few contacts: the whole solve in one block's shared memory ----
+// Up to kSmallContacts contacts whose nodes fit in shared memory are solved by
+// one block alone, with the phases and the arithmetic of solve_body. What costs
+// the cluster its 21 us per iteration at 300 contacts is not work but round
+// trips: gathers from L2, reductions into it, a cluster barrier after each
+// phase. Here a thread owns a contact (geometry, stencil weights, velocity and
+// line form in registers) and every kThreads-th node, nodes and per-contact
+// derivatives lie in shared memory, and phases end in __syncthreads:
+//   - the contact nodes get numbers through a hash table of their addresses
+//     that keeps a 4^3 block's nodes together, so that the threads of a warp
+//     own neighbours;
+//   - phase G gathers v_c through the contact's 27 node numbers;
+//   - phase N sums each node's contact terms over its list of (contact,
+//     weight) pairs (compressed rows, built once), no reductions in memory;
+//   - warp 0 sums the warps' partial sums, tests and picks the next points
+//     itself, while the other warps form dv_c.
+// Bound by latency: chains of shared-memory round trips (list rows in N, the
+// contact's nodes in G and C) and the line search's scalar step. Measured: a
+// quasi-Newton iteration of 288 contacts and 486 nodes 21.5 -> 13.3 us (G 2.7,
+// N 4.5, C and 3.1 passes 6.1), a substep of 15 contacts without iterations
+// 18.6 -> 10.3 us, a solve of 60 contacts at eps_r = 1e-5 235 -> 95 us. At 400
+// contacts with one iteration per substep it gains nothing over the cluster
+// (37 us and a launch against 45 us): the line is at 320.
+// A kernel of its own, before the cluster's: the registers and the 204 KB of
+// shared memory that it wants would slow the general path down (with them, the
+// node list alone of 3,100 contacts took the cluster 43 instead of 17 us).
+// It sets a flag that the other solve kernels of the substep test.
+constexpr int kSmallContacts = 320;
+constexpr int kSmallFlag = 16;      // word of SolveArgs::bar: 1 if the one-block kernel solved the substep
+constexpr int kSmallHash = 8192;    // slots of the node hash table (128 blocks of 64)
+constexpr int kSmallNodes = 4096;   // most nodes (half of the table)
+constexpr int kSmallProbes = 32;
+constexpr size_t kSmallSmem = 204 * 1024;
+
+__device__ __forceinline__ size_t small_bytes(int nc, int nn) {  // as small_solve lays it out
+  return (size_t)nn * 60 + (size_t)nc * (36 + 27 * 6) + ((nc + 1) & ~1) * (27 * 2 + 48) + 256;
+}
+
+// exclusive prefix sum of v over the block's threads, and its total
+__device__ __forceinline__ int block_scan(int v, int* s_warp, int& total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_warp[w] = x;
+  __syncthreads();
+  int t = lane < kWarps ? s_warp[lane] : 0;
+#pragma unroll
+  for (int o = 1; o < kWarps; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, t, o);
+    if (lane >= o) t += y;
+  }
+  total = __shfl_sync(0xffffffffu, t, kWarps - 1);
+  const int before = __shfl_sync(0xffffffffu, t, w > 0 ? w - 1 : 0);
+  __syncthreads();
+  return (w > 0 ? before : 0) + x - v;
+}
+
+// slots of the three nodes of a stencil row in the hash table (inserted if
+// new); false if one finds none. A node's 4^3 block picks a run of 64 slots,
+// probed in order; the three first probes are in flight together.
+__device__ __forceinline__ bool small_slots(int* keys, const int (&node)[3], int (&slot)[3]) {
+  int old[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    slot[k] = (int)((((unsigned)(node[k] >> 6) * 2654435761u) >> 25) * 64 + (node[k] & 63));
+    old[k] = atomicCAS(keys + slot[k], -1, node[k]);
+  }
+  bool ok = true;
+#pragma unroll 1
+  for (int probe = 0; probe < kSmallProbes; ++probe) {
+    bool more = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (old[k] != -1 && old[k] != node[k]) {
+        slot[k] = (slot[k] + 64) & (kSmallHash - 1);
+        old[k] = atomicCAS(keys + slot[k], -1, node[k]);
+        more = true;
+      }
+    if (!more) break;
+    ok = probe + 1 < kSmallProbes;
+  }
+  return ok;
+}
+
+// The substep's solve by this block if it has at most kSmallContacts contacts
+// whose nodes fit; the flag says whether.
+__device__ __forceinline__ void small_solve(const SolveArgs& a) {
+  __shared__ DevBody s_body[kMaxBodies];
+  __shared__ float s_red[kWarps][kRedWidth];
+  __shared__ float s_imp[kMaxBodies][6];
+  __shared__ float s_pts[kLsPoints];
+  __shared__ float2 s_A, s_B;
+  __shared__ float s_alpha;
+  __shared__ int s_dec;
+  extern __shared__ float4 s_line[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(s_line);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int* s_warp = reinterpret_cast<int*>(&s_red[0][0]);
+  const int count = *a.C.count;
+  const int nc = count < a.C.cap ? count : a.C.cap;
+  if (nc == 0 || nc > a.small_max || __ldcg(a.poison)) {
+    if (tid == 0) a.bar[kSmallFlag] = 0u;
+    return;
+  }
+  for (int i = tid; i < a.nb * (int)(sizeof(DevBody) / 4); i += kThreads)
+    reinterpret_cast<float*>(s_body)[i] = reinterpret_cast<const float*>(a.bodies)[i];
+  for (int i = tid; i < kMaxBodies * 6; i += kThreads) (&s_imp[0][0])[i] = 0.f;
+  __syncthreads();
+
+  PhaseClock clk;
+  if (tid == 0) clk.start();
+  auto lap = [&](int ph) {
+    if (tid == 0) clk.lap(ph);
+  };
+
+  // this thread's contact
+  const bool own = tid < nc;
+  float4 xp = make_float4(0.f, 0.f, 0.f, 0.f);
+  float n[3] = {0.f, 0.f, 1.f}, n0 = 0.f, bias[3] = {0.f, 0.f, 0.f};
+  int body = 0;
+  if (own) {
+    load_contact(a.C, tid, xp, n, n0);
+    const float4 b = a.C.bias[tid];
+    bias[0] = b.x; bias[1] = b.y; bias[2] = b.z;
+    body = a.C.id[tid].y;
+  }
+  const DevBody& bd = s_body[body];
+  // the contact's stencil, a row of three nodes at a time: rolled loops (the
+  // row's weights rotate) keep the kernel's code small, and with one or two
+  // iterations per substep it is fetched cold
+  float wx[3] = {}, wy[3] = {}, wz[3] = {};
+  auto for_nodes = [&](auto f) {
+#pragma unroll 1
+    for (int cz = 0; cz < 3; ++cz) {
+#pragma unroll 1
+      for (int cy = 0; cy < 3; ++cy) {
+#pragma unroll
+        for (int cx = 0; cx < 3; ++cx) f(9 * cz + 3 * cy + cx, wx[cx] * wy[0] * wz[0], cx, cy, cz);
+        const float y0 = wy[0];
+        wy[0] = wy[1];
+        wy[1] = wy[2];
+        wy[2] = y0;
+      }
+      const float z0 = wz[0];
+      wz[0] = wz[1];
+      wz[1] = wz[2];
+      wz[2] = z0;
+    }
+  };
+  // setup work on rows of three nodes: with few contacts several threads share
+  // a contact's nine rows (thread `part` of `parts`, contact `ct`)
+  const int ncw = (nc + 31) & ~31, parts = kThreads / ncw, part = tid / ncw;
+  const int ct = tid - part * ncw;
+  const bool rows = ct < nc && part < parts;
+  const int ncp = (nc + 1) & ~1;
+  uint16_t* ids = reinterpret_cast<uint16_t*>(smem);  // [27][ncp]: the contacts' node numbers
+  auto number = [&](int c) { return (int)ids[c * ncp + tid]; };
+  float* cw = reinterpret_cast<float*>(smem + ((size_t)27 * ncp * 2 + 15) / 16 * 16);  // weights (9), base (3)
+  int* gnode = reinterpret_cast<int*>(cw + ((12 * ncp + 3) & ~3));                     // the nodes' addresses
+  int nn = 0;
+  {
+    // node numbers: hash table slots, then the order of the occupied slots
+    int* keys = reinterpret_cast<int*>(smem + kSmallSmem - kSmallHash * 6);
+    uint16_t* vals = reinterpret_cast<uint16_t*>(keys + kSmallHash);
+    for (int i = tid; i < kSmallHash / 4; i += kThreads)
+      reinterpret_cast<int4*>(keys)[i] = make_int4(-1, -1, -1, -1);
+    if (own) {
+      Stencil st;
+      stencil(a.g, xp.x, xp.y, xp.z, st);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        wx[k] = st.w[0][k];
+        wy[k] = st.w[1][k];
+        wz[k] = st.w[2][k];
+        cw[k * ncp + tid] = wx[k];
+        cw[(3 + k) * ncp + tid] = wy[k];
+        cw[(6 + k) * ncp + tid] = wz[k];
+        reinterpret_cast<int*>(cw)[(9 + k) * ncp + tid] = st.base[k];
+      }
+    }
+    __syncthreads();
+    bool fits = true;
+    if (rows) {
+      const int* base = reinterpret_cast<const int*>(cw) + 9 * ncp + ct;
+      const int bx = base[0], by = base[ncp], bz = base[2 * ncp];
+#pragma unroll 1
+      for (int r = part; r < 9; r += parts) {
+        int node[3], slot[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) node[k] = node_index(a.g, bx + k, by + r % 3, bz + r / 3);
+        fits = small_slots(keys, node, slot) && fits;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) ids[(3 * r + k) * ncp + ct] = (uint16_t)slot[k];
+      }
+    }
+    fits = __syncthreads_and(fits);
+    // a warp numbers kSmallHash / kWarps consecutive slots, 32 at a time
+    constexpr int kRuns = kSmallHash / kThreads;
+    const int slot0 = warp * (kSmallHash / kWarps) + lane;
+    int count = 0;
+#pragma unroll 4
+    for (int j = 0; j < kRuns; ++j) count += __popc(__ballot_sync(0xffffffffu, keys[slot0 + 32 * j] >= 0));
+    if (lane == 0) s_warp[warp] = count;
+    __syncthreads();
+    int id = 0;
+#pragma unroll 4
+    for (int w = 0; w < kWarps; ++w) {
+      const int c = s_warp[w];
+      id += w < warp ? c : 0;
+      nn += c;
+    }
+    __syncthreads();
+    fits = fits && nn <= kSmallNodes && small_bytes(nc, nn) <= kSmallSmem;
+    if (tid == 0) a.bar[kSmallFlag] = fits ? 1u : 0u;
+    if (!fits) return;
+    // (the list in memory serves the tape)
+#pragma unroll 2
+    for (int j = 0; j < kRuns; ++j) {
+      const int key = keys[slot0 + 32 * j];
+      const unsigned used = __ballot_sync(0xffffffffu, key >= 0);
+      if (key >= 0) {
+        const int k = id + __popc(used & ((1u << lane) - 1u));
+        vals[slot0 + 32 * j] = (uint16_t)k;
+        gnode[k] = key;
+        if (k < a.G.cnodes_cap) a.G.cnodes[k] = key;
+      }
+      id += __popc(used);
+    }
+    if (tid == 0) *a.G.n_cnodes = nn;
+    __syncthreads();
+    if (rows)
+#pragma unroll 1
+      for (int r = part; r < 9; r += parts)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          uint16_t* id3 = ids + (3 * r + k) * ncp + ct;
+          *id3 = vals[*id3];
+        }
+    __syncthreads();
+  }
+  // shared memory: node state, contact terms, rows
+  unsigned char* at = reinterpret_cast<unsigned char*>(gnode) + ((size_t)nn * 4 + 15) / 16 * 16;
+  auto take = [&](size_t bytes) {
+    unsigned char* p = at;
+    at += (bytes + 15) / 16 * 16;
+    return p;
+  };
+  float4* nvs = reinterpret_cast<float4*>(take((size_t)nn * 16));  // (v*, m), m < 0: not a free DoF
+  float4* nva = reinterpret_cast<float4*>(take((size_t)nn * 16));  // (v hi, v lo x)
+  float2* nvb = reinterpret_cast<float2*>(take((size_t)nn * 8));   // (v lo y, z)
+  float* ndv = reinterpret_cast<float*>(take((size_t)nn * 12));    // search direction, three planes
+  int* off = reinterpret_cast<int*>(take((size_t)nn * 4));         // rows' starts, then ends
+  float4* rec0 = reinterpret_cast<float4*>(take((size_t)nc * 16)); // (g, Hxx)
+  float4* rec1 = reinterpret_cast<float4*>(take((size_t)nc * 16)); // (Hyy, Hzz, Hxy, Hxz)
+  float* rec2 = reinterpret_cast<float*>(take((size_t)nc * 4));    // Hyz
+  float* ew = reinterpret_cast<float*>(take((size_t)27 * nc * 4));
+  uint16_t* ec = reinterpret_cast<uint16_t*>(take((size_t)27 * nc * 2));
+  // the nodes: v, v* (the iterate's low part starts at zero, as the grid
+  // update leaves it)
+  for (int i = tid; i < nn; i += kThreads) {
+    const int gn = gnode[i];
+    const float4 v = a.G.v[gn], vs = a.G.vs[gn];
+    const bool free_dof = vs.w > 0.f && v.w == 0.f;
+    nvs[i] = make_float4(vs.x, vs.y, vs.z, free_dof ? vs.w : -1.f);
+    nva[i] = make_float4(v.x, v.y, v.z, 0.f);
+    nvb[i] = make_float2(0.f, 0.f);
+    off[i] = 0;
+  }
+  __syncthreads();
+  // rows: a node's (contact, weight) pairs
+  if (rows)
+#pragma unroll 1
+    for (int r = part; r < 9; r += parts)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) atomicAdd(off + ids[(3 * r + k) * ncp + ct], 1);
+  __syncthreads();
+  {
+    const int per = (nn + kThreads - 1) / kThreads, i0 = min(tid * per, nn), i1 = min(i0 + per, nn);
+    int sum = 0;
+    for (int i = i0; i < i1; ++i) sum += off[i];
+    int total = 0;
+    int start = block_scan(sum, s_warp, total);
+    for (int i = i0; i < i1; ++i) {
+      const int cnt = off[i];
+      off[i] = start;
+      start += cnt;
+    }
+  }
+  __syncthreads();
+  if (rows)
+#pragma unroll 1
+    for (int r = part; r < 9; r += parts) {
+      const float y = cw[(3 + r % 3) * ncp + ct], z = cw[(6 + r / 3) * ncp + ct];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int pos = atomicAdd(off + ids[(3 * r + k) * ncp + ct], 1);
+        ec[pos] = (uint16_t)ct;
+        ew[pos] = cw[k * ncp + ct] * y * z;
+      }
+    }
+  // (off[i] ends as row i's end: row i starts at off[i - 1])
+  const double pstar2_d = __ldcg(a.G.pstar2);
+  const float pstar2_hi = (float)pstar2_d, pstar2_lo = (float)(pstar2_d - (double)pstar2_hi);
+  const float eps_a = (float)a.eps_a, eps_r = (float)a.eps_r;
+  lap(0);
+
+  LineSearch ls;  // used by warp 0
+  float u[3] = {0.f, 0.f, 0.f}, dvc[3] = {0.f, 0.f, 0.f};
+  float alpha = 0.f, resid = 0.f;
+  int it = 0, ls_passes = 0;
+  for (;;) {
+    // ---- G
+    if (own) {
+      float S[3] = {0.f, 0.f, 0.f}, E[3] = {0.f, 0.f, 0.f};
+      for_nodes([&](int c, float w, int, int, int) {
+        const int id = number(c);
+        const float4 q = nva[id];
+        const float2 r = nvb[id];
+        const float hv[3] = {q.x, q.y, q.z}, lv[3] = {q.w, r.x, r.y};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float pr = w * hv[k];
+          const float pe = fmaf(w, hv[k], -pr) + w * lv[k];
+          float sum, err;
+          two_sum(S[k], pr, sum, err);
+          S[k] = sum;
+          E[k] += err + pe;
+        }
+      });
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        CompSum cs;
+        cs.S = S[k] + E[k];
+        cs.add(bias[k]);
+        cs.add_prod(alpha, dvc[k]);
+        u[k] = cs.value();
+      }
+      ContactLaw L;
+      contact_law(xp.w, n0, bd.mu, bd.k, bd.d, a.h, a.eps_s, n, u, L);
+      float gr[3], H[6];
+      contact_grad(L, n, gr);
+      contact_hess(L, n, H);
+      rec0[tid] = make_float4(gr[0], gr[1], gr[2], H[0]);
+      rec1[tid] = make_float4(H[1], H[2], H[3], H[4]);
+      rec2[tid] = H[5];
+    }
+    __syncthreads();
+    lap(1);
+
+    // ---- N
+    float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // G2, P2 - P*2, J2, A, B
+    for (int i = tid; i < nn; i += kThreads) {
+      const float4 vs = nvs[i];
+      float dx = 0.f, dy = 0.f, dz = 0.f;
+      if (vs.w > 0.f) {  // free DoF
+        float4 v = nva[i];
+        float2 vl = nvb[i];
+        if (it > 0) {
+          dd_add(v.x, v.w, alpha * ndv[i]);
+          dd_add(v.y, vl.x, alpha * ndv[nn + i]);
+          dd_add(v.z, vl.y, alpha * ndv[2 * nn + i]);
+          nva[i] = v;
+          nvb[i] = vl;
+        }
+        float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+        float c2 = 0.f;
+        const int end = off[i];
+#pragma unroll 2
+        for (int e = i > 0 ? off[i - 1] : 0; e < end; ++e) {
+          const int c = ec[e];
+          const float w = ew[e], w2 = w * w;
+          const float4 q0 = rec0[c], q1 = rec1[c];
+          c0.x = fmaf(w, q0.x, c0.x);
+          c0.y = fmaf(w, q0.y, c0.y);
+          c0.z = fmaf(w, q0.z, c0.z);
+          c0.w = fmaf(w2, q0.w, c0.w);
+          c1.x = fmaf(w2, q1.x, c1.x);
+          c1.y = fmaf(w2, q1.y, c1.y);
+          c1.z = fmaf(w2, q1.z, c1.z);
+          c1.w = fmaf(w2, q1.w, c1.w);
+          c2 = fmaf(w2, rec2[c], c2);
+        }
+        const float r0 = (v.x - vs.x) + v.w, r1 = (v.y - vs.y) + vl.x, r2 = (v.z - vs.z) + vl.y;
+        node_step(vs.w, vs, r0, r1, r2, c0, c1, c2, dx, dy, dz, acc);
+      }
+      ndv[i] = dx;
+      ndv[nn + i] = dy;
+      ndv[2 * nn + i] = dz;
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const float t = warp_sum(acc[k]);
+      if (lane == 0) s_red[warp][k] = t;
+    }
+    __syncthreads();
+    lap(2);
+    if (warp == 0) {
+      // totals of the warps' sums: lane l takes value l & 7 of warps l >> 3,
+      // + 4, ... (compensated)
+      const int k = lane & 7;
+      float S = 0.f, E = 0.f;
+#pragma unroll
+      for (int w = 0; w < kWarps; w += 4)
+        df_acc(S, E, make_float2(k < 5 ? s_red[w + (lane >> 3)][k] : 0.f, 0.f));
+#pragma unroll
+      for (int o = 8; o < 32; o <<= 1) {
+        const float S2 = __shfl_xor_sync(0xffffffffu, S, o), E2 = __shfl_xor_sync(0xffffffffu, E, o);
+        float s2, e;
+        two_sum(S, S2, s2, e);
+        S = s2;
+        E = E + E2 + e;
+      }
+      const float2 mine = df_norm(S, E);
+      float2 tot[5];
+#pragma unroll
+      for (int q = 0; q < 5; ++q)
+        tot[q] = make_float2(__shfl_sync(0xffffffffu, mine.x, q), __shfl_sync(0xffffffffu, mine.y, q));
+      if (lane == 0) {
+        s_dec = stop_test(a, tot, pstar2_hi, pstar2_lo, eps_a, eps_r, it, true, resid);
+        s_A = tot[3];
+        s_B = tot[4];
+      }
+      ls.reset();
+      if (lane < kLsPoints) s_pts[lane] = ls.pt;
+    }
+    // ---- C: dv_c = J dv and the contact's line form
+    ContactLine line = ContactLine{};
+    if (own) {
+      float e[3] = {0.f, 0.f, 0.f};
+      for_nodes([&](int c, float w, int, int, int) {
+        const int id = number(c);
+        e[0] = fmaf(w, ndv[id], e[0]);
+        e[1] = fmaf(w, ndv[nn + id], e[1]);
+        e[2] = fmaf(w, ndv[2 * nn + id], e[2]);
+      });
+#pragma unroll
+      for (int k = 0; k < 3; ++k) dvc[k] = e[k];
+      contact_line(xp.w, n0, bd.mu, bd.k, bd.d, a.h, a.eps_s, n, u, e, line);
+    }
+    __syncthreads();
+    if (s_dec) break;
+    // ---- L
+    for (int pass = 0;; ++pass) {
+      float v16[16];
+#pragma unroll
+      for (int j = 0; j < 2 * kLsPoints; ++j) v16[j] = 0.f;
+      if (own) {
+#pragma unroll
+        for (int j = 0; j < kLsPoints; j += 2) {
+          float2 d1, d2;
+          contact_line_eval2(line, make_float2(s_pts[j], s_pts[j + 1]), d1, d2);
+          v16[j] = d1.x;
+          v16[j + 1] = d1.y;
+          v16[kLsPoints + j] = d2.x;
+          v16[kLsPoints + j + 1] = d2.y;
+        }
+      }
+      const float t = warp_sums16(v16, lane);
+      if (lane < 16) s_red[warp][lane] = t;
+      __syncthreads();
+      ++ls_passes;
+      if (warp == 0) {
+        // lane l: value l & 15 of warps l >> 4, + 2, ...
+        float S = 0.f, E = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; w += 2)
+          df_acc(S, E, make_float2(s_red[w + (lane >> 4)][lane & 15], 0.f));
+        const float S2 = __shfl_xor_sync(0xffffffffu, S, 16), E2 = __shfl_xor_sync(0xffffffffu, E, 16);
+        float s2, e;
+        two_sum(S, S2, s2, e);
+        const float2 mine = df_norm(s2, E + E2 + e);
+        const int k = lane & (kLsPoints - 1);
+        const float2 tk = make_float2(__shfl_sync(0xffffffffu, mine.x, k), __shfl_sync(0xffffffffu, mine.y, k));
+        const float2 tk2 = make_float2(__shfl_sync(0xffffffffu, mine.x, kLsPoints + k),
+                                       __shfl_sync(0xffffffffu, mine.y, kLsPoints + k));
+        const int state = ls.update(tk, tk2, s_A, s_B, a.ls_rel_tol, pass + 1 >= a.ls_max_iters);
+        if (lane == 0) {
+          if (state == LineSearch::kFailed) atomicOr(a.status, kStLineSearch);
+          s_dec = state != LineSearch::kMore;
+          s_alpha = ls.best;
+        }
+        if (lane < kLsPoints) s_pts[lane] = ls.pt;
+      }
+      __syncthreads();
+      if (s_dec) break;
+    }
+    lap(3);
+    alpha = s_alpha;
+    ++it;
+    if (alpha == 0.f) break;
+  }
+  // the solution to G.v, which G2P reads (the other nodes keep v = v*)
+  for (int i = tid; i < nn; i += kThreads) {
+    if (nvs[i].w > 0.f) {
+      const float4 v = nva[i];
+      a.G.v[gnode[i]] = make_float4(v.x, v.y, v.z, 0.f);
+    }
+  }
+  // impulses at the solution
+  if (own) a.C.vc[tid] = make_float4(u[0], u[1], u[2], 0.f);
+  contact_impulses(a, s_body, tid, own, xp, n, n0, body, u, lane, s_imp);
+  __syncthreads();
+  for (int i = tid; i < a.nb * 6; i += kThreads) {
+    const float v = (&s_imp[0][0])[i];
+    if (v != 0.f) atomicAdd(a.impulses + i, (double)v);
+  }
+  lap(4);
+  if (tid == 0) {
+    clk.finish();
+    solve_stats(a, clk.t, it, ls_passes, false, true, nn, resid);
+  }
+}
+
 // kCluster: the solve of up to a.cluster_max contacts by the blocks of one
 // thread-block cluster (hardware cluster barriers, block sums exchanged
 // through distributed shared memory); otherwise the cooperative launch over
@@ -491,6 +1137,7 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   const int nc = count < a.C.cap ? count : a.C.cap;
   if (nc == 0) return;  // v = v* already (set by the grid update)
   // (every block of a launch reads the same count: the choice is uniform)
+  if (nc <= a.small_max && __ldcg(a.bar + kSmallFlag)) return;  // solved by the one-block kernel
   if (kCluster ? nc > a.cluster_max : nc <= a.cluster_max) return;  // the other kernel's
   int nblk = grid_blocks;  // a cluster: all of its blocks
   if (!kCluster) {
@@ -506,14 +1153,10 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   __syncthreads();
 
   // phase timers (block 0, thread 0): list, G, N, line search, impulses
-  unsigned long long tph[5] = {0ull, 0ull, 0ull, 0ull, 0ull};
-  unsigned long long tmark = global_ns();
+  PhaseClock clk;
+  if (block == 0 && tid == 0) clk.start();
   auto lap = [&](int ph) {
-    if (block == 0 && tid == 0) {
-      const unsigned long long now = global_ns();
-      tph[ph] += now - tmark;
-      tmark = now;
-    }
+    if (block == 0 && tid == 0) clk.lap(ph);
   };
   // (wait_extra > 0 only in the test of the barrier's time limit: the
   // barrier then waits for arrivals that never come)
@@ -768,28 +1411,7 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
         if (m > 0.f && v.w == 0.f) {  // free DoF (v.w flags a Dirichlet node)
           // v - v* with the low part of the iterate
           const float r0 = (v.x - vs.x) + vl.x, r1 = (v.y - vs.y) + vl.y, r2 = (v.z - vs.z) + vl.z;
-          const float g0 = m * r0 + c0.x, g1 = m * r1 + c0.y, g2 = m * r2 + c0.z;
-          const float inv_m = 1.0f / m;
-          acc[0] += (g0 * g0 + g1 * g1 + g2 * g2) * inv_m;
-          // m (|v|^2 - |v*|^2) = m r . (2 v* + r)
-          acc[1] += m * (r0 * (2.f * vs.x + r0) + r1 * (2.f * vs.y + r1) + r2 * (2.f * vs.z + r2));
-          acc[2] += (c0.x * c0.x + c0.y * c0.y + c0.z * c0.z) * inv_m;
-          // H = m I + contact block; dv = -H^-1 g (Cholesky)
-          const float h00 = m + c0.w, h11 = m + c1.x, h22 = m + c1.y;
-          const float h01 = c1.z, h02 = c1.w, h12 = c2;
-          const float l00 = sqrtf(h00);
-          const float l10 = h01 / l00, l20 = h02 / l00;
-          const float l11 = sqrtf(fmaxf(h11 - l10 * l10, 1e-30f));
-          const float l21 = (h12 - l20 * l10) / l11;
-          const float l22 = sqrtf(fmaxf(h22 - l20 * l20 - l21 * l21, 1e-30f));
-          const float y0 = -g0 / l00;
-          const float y1 = (-g1 - l10 * y0) / l11;
-          const float y2 = (-g2 - l20 * y0 - l21 * y1) / l22;
-          dv.z = y2 / l22;
-          dv.y = (y1 - l21 * dv.z) / l11;
-          dv.x = (y0 - l10 * dv.y - l20 * dv.z) / l00;
-          acc[3] += m * (dv.x * dv.x + dv.y * dv.y + dv.z * dv.z);
-          acc[4] += m * (dv.x * r0 + dv.y * r1 + dv.z * r2);
+          node_step(m, vs, r0, r1, r2, c0, c1, c2, dv.x, dv.y, dv.z, acc);
         }
         a.G.dv[node] = dv;
       }
@@ -805,25 +1427,9 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
     // (FP64 is a narrow pipe on GB300) and the decision is broadcast; every
     // block computes it from the same totals, so all decide alike.
     if (tid == 0) {
-      const float2 A = s_tot[3], Bs = s_tot[4];
-      const float G2 = s_tot[0].x + s_tot[0].y, J2 = s_tot[2].x + s_tot[2].y;
-      const float P2 = (pstar2_hi + s_tot[1].x) + (pstar2_lo + s_tot[1].y);
-      const float Gn = sqrtf(G2), Pn = sqrtf(fmaxf(P2, 0.f)), Jn = sqrtf(J2);
-      const float mx = fmaxf(Pn, Jn);
-      resid = mx > 0.f ? Gn / mx : 0.f;
-      int dec = 0;
-      if (!(G2 == G2) || !(A.x == A.x) || !(Bs.x == Bs.x)) {
-        if (block == 0) atomicOr(a.status, kStNan);
-        dec = 1;
-      } else if (Gn < eps_a + eps_r * mx || G2 == 0.f) {
-        dec = 1;  // converged
-      } else if (it >= a.max_iters) {
-        if (block == 0) atomicOr(a.status, kStNotConverged);
-        dec = 1;
-      }
-      s_dec = dec;
-      s_A = A;
-      s_B = Bs;
+      s_dec = stop_test(a, s_tot, pstar2_hi, pstar2_lo, eps_a, eps_r, it, block == 0, resid);
+      s_A = s_tot[3];
+      s_B = s_tot[4];
     }
     if (tid < 32) {
       ls.reset();
@@ -890,18 +1496,21 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
           if (k < kLsCacheDepth) line_store(s_line, slot, L, b);
         }
 #pragma unroll
-        for (int j = 0; j < kLsPoints; ++j) {
-          float d1, d2;
-          contact_line_eval(L, alphas[j], d1, d2);
-          acc[j] += d1;
-          acc[kLsPoints + j] += d2;
+        for (int j = 0; j < kLsPoints; j += 2) {
+          float2 d1, d2;
+          contact_line_eval2(L, make_float2(alphas[j], alphas[j + 1]), d1, d2);
+          acc[j] += d1.x;
+          acc[j + 1] += d1.y;
+          acc[kLsPoints + j] += d2.x;
+          acc[kLsPoints + j + 1] += d2.y;
         }
       }
       if (!reduce_all(acc, sl, local_ls ? Bl : B, s_red, s_tot, local_ls ? nullptr : next_cpart()))
         return;
       ++ls_passes;
       if (tid < 32) {
-        const int st = ls.update(s_tot, s_A, s_B, a.ls_rel_tol, pass + 1 >= a.ls_max_iters);
+        const int st = ls.update(s_tot[tid & (kLsPoints - 1)], s_tot[kLsPoints + (tid & (kLsPoints - 1))],
+                                 s_A, s_B, a.ls_rel_tol, pass + 1 >= a.ls_max_iters);
         if (tid == 0) {
           if (st == LineSearch::kFailed && block == 0) atomicOr(a.status, kStLineSearch);
           s_dec = st != LineSearch::kMore;
@@ -931,43 +1540,16 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   // each warp sums its contacts body by body before the block's shared sums
   for (int p0 = gtid & ~31; p0 < nc; p0 += gstride) {
     const int p = p0 + lane;
-    int b = -1;
-    float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float4 xp = make_float4(0.f, 0.f, 0.f, 0.f), vc = xp;
+    float n[3] = {0.f, 0.f, 1.f}, n0 = 0.f;
+    int body = 0;
     if (p < nc) {
-      float4 xp; float n[3]; float n0;
       load_contact(a.C, p, xp, n, n0);
-      b = a.C.id[p].y;
-      const DevBody& bd = s_body[b];
-      const float4 vc = __ldcg(a.C.vc + p);
-      const float u[3] = {vc.x, vc.y, vc.z};
-      ContactLaw L;
-      contact_law(xp.w, n0, bd.mu, bd.k, bd.d, a.h, a.eps_s, n, u, L);
-      float gr[3];
-      contact_grad(L, n, gr);
-      a.C.gamma[p] = make_float4(-gr[0], -gr[1], -gr[2], 0.f);
-      const float r0 = xp.x - bd.p[0], r1 = xp.y - bd.p[1], r2 = xp.z - bd.p[2];
-      q[0] = gr[0]; q[1] = gr[1]; q[2] = gr[2];
-      q[3] = r1 * gr[2] - r2 * gr[1];
-      q[4] = r2 * gr[0] - r0 * gr[2];
-      q[5] = r0 * gr[1] - r1 * gr[0];
+      body = a.C.id[p].y;
+      vc = __ldcg(a.C.vc + p);
     }
-    unsigned left = __ballot_sync(0xffffffffu, b >= 0);
-    while (left) {  // one body of the warp at a time (mostly a single one)
-      const int bb = __shfl_sync(0xffffffffu, b, __ffs(left) - 1);
-      const bool mine = b == bb;
-      float t[6];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        t[c] = mine ? q[c] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t[c] += __shfl_xor_sync(0xffffffffu, t[c], o);
-      }
-      if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) atomicAdd(&s_imp[bb][c], t[c]);
-      }
-      left &= ~__ballot_sync(0xffffffffu, mine);
-    }
+    const float u[3] = {vc.x, vc.y, vc.z};
+    contact_impulses(a, s_body, p, p < nc, xp, n, n0, body, u, lane, s_imp);
   }
   __syncthreads();
   for (int i = tid; i < a.nb * 6; i += kThreads) {
@@ -976,16 +1558,22 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   }
   lap(4);
   if (gtid == 0) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) atomicAdd(&a.stats->solve_ns[k], tph[k]);
-    atomicAdd(&a.stats->iters_total, it);
-    atomicMax(&a.stats->iters_max, it);
-    atomicAdd(&a.stats->ls_evals_total, ls_passes);
-    if (!local_ls) atomicAdd(&a.stats->ls_split, 1);
-    if (kCluster) atomicAdd(&a.stats->cluster, 1);
-    atomicMax(&a.stats->cnodes_max, ncn);
-    atomicMax(reinterpret_cast<int*>(&a.stats->residual_max), __float_as_int(resid));
+    clk.finish();
+    solve_stats(a, clk.t, it, ls_passes, !local_ls, kCluster, ncn, resid);
   }
+}
+
+__global__ void __launch_bounds__(kThreads, 1) k_solve_small(SolveArgs a) { small_solve(a); }
+
+// Batched: a block per scene
+__global__ void __launch_bounds__(kThreads, 1) k_solve_small_batch(const SolveArgs* __restrict__ args,
+                                                                   const int* __restrict__ order) {
+  __shared__ SolveArgs s_a;
+  load_args(args + order[blockIdx.x], s_a);
+  __syncthreads();
+  if (threadIdx.x == 0) s_a.small_max = kSmallContacts;
+  __syncthreads();
+  small_solve(s_a);
 }
 
 template <bool kCluster>
@@ -1004,7 +1592,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve_batch(const SolveArgs* __
   __shared__ SolveArgs s_a;
   load_args(args + order[blockIdx.x / kBlocks], s_a);
   __syncthreads();
-  if (threadIdx.x == 0) s_a.cluster_max = kBlocks > 1 ? 0x7fffffff : 0;  // this launch's kind
+  if (threadIdx.x == 0) {
+    s_a.cluster_max = kBlocks > 1 ? 0x7fffffff : 0;  // this launch's kind
+    s_a.small_max = kSmallContacts;
+  }
   __syncthreads();
   if constexpr (kBlocks == 1)
     solve_body<false>(s_a, 0, 1);
@@ -1798,6 +2389,10 @@ cudaError_t solve_prepare() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_solve<true>),
                              cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  for (const void* f : {reinterpret_cast<const void*>(&k_solve_small),
+                        reinterpret_cast<const void*>(&k_solve_small_batch)})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
   for (const void* f : {reinterpret_cast<const void*>(&k_solve_batch<1>),
                         reinterpret_cast<const void*>(&k_solve_batch<2>),
                         reinterpret_cast<const void*>(&k_solve_batch<4>),
@@ -1841,12 +2436,15 @@ int solve_cluster_blocks() {
 cudaError_t launch_solve(const SolveArgs& a, int grid_blocks, int cluster_blocks, cudaStream_t s) {
   SolveArgs args = a;
   if (cluster_blocks > 0 && args.cluster_max > 0) {
+    args.small_max = args.cluster_max < kSmallContacts ? args.cluster_max : kSmallContacts;
+    k_solve_small<<<1, kThreads, kSmallSmem, s>>>(args);
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = cluster_config(cluster_blocks, &attr, s);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k_solve<true>, args);
     if (e != cudaSuccess) return e;
   } else {
     args.cluster_max = 0;
+    args.small_max = 0;
   }
   void* params[] = {&args};
   return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_solve<false>),
@@ -1874,6 +2472,7 @@ cudaError_t launch_solve_batch_k(const SolveArgs* args, const int* order, int n_
 cudaError_t launch_solve_batch(const SolveArgs* args, const int* order, int n_scenes,
                                int blocks_per_scene, cudaStream_t s) {
   if (n_scenes <= 0) return cudaSuccess;
+  k_solve_small_batch<<<n_scenes, kThreads, kSmallSmem, s>>>(args, order);
   switch (blocks_per_scene) {
     case 2: return launch_solve_batch_k<2>(args, order, n_scenes, s);
     case 4: return launch_solve_batch_k<4>(args, order, n_scenes, s);
