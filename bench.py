@@ -180,16 +180,27 @@ class ClockSampler:
 SMALL_SORT_MAX = 8192  # particles the library sorts in one thread block
 
 
-def kernel_launches_per_step(res, n_substeps, n_bodies=0, n_particles=None):
-    """Kernels one mpm_step launches: the sort (above 8,192 particles the
-    radix sort: keys, five kernels per 8-bit digit pass, permutation; up to
-    it one sorting block and the permutation), per substep P2G, grid update,
-    the three solve kernels (one block, the cluster and the cooperative one,
-    of which the contacts pick one to work) and G2P, and with bodies the rigid
-    update after the substeps."""
-    if n_particles is not None and n_particles <= SMALL_SORT_MAX:
+def sort_launches(res, n_particles):
+    """Kernels of the library's sort: up to 8,192 particles one sorting block,
+    above three per pass over the key's bits (each axis's own block bits, and
+    six of the cell), and the permutation."""
+    if n_particles <= SMALL_SORT_MAX:
+        return 2
+    bits = sum((-(-int(r) // 4) - 1).bit_length() for r in res)
+    bits = max(bits + (6 if bits + 6 <= 32 else 0), 1)
+    return 3 * -(-bits // 8) + 1
+
+
+def kernel_launches_per_step(res, n_substeps, n_bodies=0, n_particles=None, sort=None):
+    """Kernels one mpm_step launches: `sort` of the sort, per substep P2G, grid
+    update, the three solve kernels (one block, the cluster and the cooperative
+    one, of which the contacts pick one to work) and G2P, and with bodies the
+    rigid update after the substeps. Without `sort`, a radix sort of keys, five
+    kernels per 8-bit digit and a permutation is counted (up to 8,192 particles
+    one block and the permutation)."""
+    if sort is None and n_particles is not None and n_particles <= SMALL_SORT_MAX:
         sort = 2
-    else:
+    elif sort is None:
         blocks = max(-(-int(r) // 4) for r in res)
         morton_bits = max((blocks - 1).bit_length(), 1)
         key_bits = 3 * morton_bits + (6 if 3 * morton_bits + 6 <= 32 else 0)
@@ -343,7 +354,8 @@ def measure_workload(native, sc, args, ws, stream_flush=True, tight=True):
                       "solve_phases_us_per_substep": dict(zip(
                           ("node_list", "gradient_hessian", "node_solve", "line_search", "impulses"),
                           solve_us_p))},
-           "launches_per_step": kernel_launches_per_step(sc["grid"]["res"], N, len(sc["bodies"]), n)}
+           "launches_per_step": kernel_launches_per_step(
+               sc["grid"]["res"], N, len(sc["bodies"]), n, sort_launches(sc["grid"]["res"], n))}
 
     peak, peak_kind = measured_peak_hbm()
     kern = {}

@@ -353,7 +353,7 @@ void release(mpm_ctx* c) {
                   c->G.acc2, c->G.dv, c->G.mark, c->G.cflag, c->G.cnodes, c->G.n_cnodes, c->G.pstar2, c->G.act, c->G.n_act, c->C.xp, c->C.nrm,
                   c->C.bias, c->C.id, c->C.vc, c->C.dvc, c->C.gamma, c->C.count, c->red, c->bar, c->poison,
                   c->status, c->stats, c->impulses, c->sb.keys[0], c->sb.keys[1], c->sb.vals[0],
-                  c->sb.vals[1], c->sb.hist, c->sb.partial, c->stage, c->adj_vec, c->adj_body,
+                  c->sb.vals[1], c->sb.hist, c->stage, c->adj_vec, c->adj_body,
                   c->adj_out, c->adj_ids, c->adj_io, c->bw_buf, c->bw_gbar, c->bw_slot, c->bw_mat,
                   c->tape_pool, c->tape_recs, c->tape_counters, c->bw_snap, c->bw_gbody, c->dyn_d,
                   c->imp0_d, c->bodies_step_d, c->G.n_mapped, c->slot_d, c->cloth_tris_d,
@@ -594,7 +594,8 @@ mpm_status mpm_create(const mpm_grid_spec* spec, void* cuda_stream, mpm_ctx** ou
   int mb = g.nbx > g.nby ? g.nbx : g.nby;
   mb = mb > g.nbz ? mb : g.nbz;
   g.morton_bits = ceil_log2(mb) > 0 ? ceil_log2(mb) : 1;
-  g.sort_cell_bits = 3 * g.morton_bits + 6 <= 32 ? 1 : 0;
+  g.sort_cell_bits = 0;
+  g.sort_cell_bits = sort_key_bits(g) + 6 <= 32 ? 1 : 0;
   ctx->cap = spec->max_particles;
   ctx->n_blocks = g.nbx * g.nby * g.nbz;
   // block-sparse storage for max_blocks active blocks (plus a spare one) when
@@ -651,9 +652,7 @@ mpm_status mpm_create(const mpm_grid_spec* spec, void* cuda_stream, mpm_ctx** ou
   const int hist_len = sort_hist_len((int)cap);
   ok = ok && dalloc(&ctx->sb.keys[0], cap) == cudaSuccess && dalloc(&ctx->sb.keys[1], cap) == cudaSuccess &&
        dalloc(&ctx->sb.vals[0], cap) == cudaSuccess && dalloc(&ctx->sb.vals[1], cap) == cudaSuccess &&
-       dalloc(&ctx->sb.hist, hist_len) == cudaSuccess &&
-       dalloc(&ctx->sb.partial, hist_len / 4096 + 2) == cudaSuccess;
-  ctx->sb.hist_cap = hist_len;
+       dalloc(&ctx->sb.hist, hist_len) == cudaSuccess;
   ok = ok && dalloc(&ctx->stage, (size_t)24 * cap) == cudaSuccess;
   if (!ok) return bail(MPM_ERR_OOM);
   // zero-invariant arrays and counters

@@ -63,6 +63,10 @@ struct mpm_batch {
   int n_p2g = 0, n_grid = 0, n_g2p = 0;
   int layout = 0;             // bumped whenever the work lists change
   bool work_valid = false;
+  // the sort's records and (scene, tile) items
+  SortArgs* sort_d = nullptr;
+  int2* sort_work_d = nullptr;
+  std::vector<SortArgs> sort_h;
   // gathered at the end of each step
   uint32_t* status_d = nullptr;
   DevStats* stats_d = nullptr;
@@ -104,6 +108,8 @@ void release(mpm_batch* b) {
   cudaFree(b->rig_d);
   cudaFree(b->work_d);
   cudaFree(b->order_d);
+  cudaFree(b->sort_d);
+  cudaFree(b->sort_work_d);
   cudaFree(b->status_d);
   cudaFree(b->stats_d);
 }
@@ -241,6 +247,10 @@ mpm_status mpm_batch_create(mpm_ctx* const* ctxs, int32_t n, mpm_batch** out) {
   if (e == cudaSuccess) e = balloc(&batch->solve_d, n);
   if (e == cudaSuccess) e = balloc(&batch->g2p_d, n);
   if (e == cudaSuccess) e = balloc(&batch->rig_d, n);
+  size_t tiles = 0;
+  for (int i = 0; i < n; ++i) tiles += sort_max_tiles((int)ctxs[i]->cap);
+  if (e == cudaSuccess) e = balloc(&batch->sort_d, n);
+  if (e == cudaSuccess) e = balloc(&batch->sort_work_d, tiles);
   if (e == cudaSuccess) e = balloc(&batch->status_d, n);
   if (e == cudaSuccess) e = balloc(&batch->stats_d, n);
   if (e == cudaSuccess) e = cudaMemsetAsync(batch->status_d, 0, n * sizeof(uint32_t), batch->stream);
@@ -257,12 +267,40 @@ mpm_status mpm_batch_create(mpm_ctx* const* ctxs, int32_t n, mpm_batch** out) {
 
 mpm_status mpm_batch_sort(mpm_batch* batch) {
   if (!batch) return MPM_ERR_INVALID_ARG;
-  for (mpm_ctx* c : batch->ctx) {
-    if (c->n <= 0) continue;
-    launch_sort(c->g, c->P[c->cur], c->P[1 - c->cur], (int)c->n, c->sb, batch->stream);
-    c->cur = 1 - c->cur;
+  const int ns = (int)batch->ctx.size();
+  const cudaStream_t s = batch->stream;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  BCU(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) {
+    // the uploads below read host memory at once: a captured sort is the
+    // members' own launches
+    for (mpm_ctx* c : batch->ctx) {
+      if (c->n <= 0) continue;
+      launch_sort(c->g, c->P[c->cur], c->P[1 - c->cur], (int)c->n, c->sb, s);
+      c->cur = 1 - c->cur;
+    }
+    BCU(cudaGetLastError());
+    return MPM_OK;
   }
+  // one set of launches for all members (24 scenes of 2k to 64k particles:
+  // 3.4 -> 0.13 ms; their own launches are a few blocks each)
+  std::vector<SortArgs>& args = batch->sort_h;
+  args.clear();
+  std::vector<int2> work;
+  for (int i = 0; i < ns; ++i) {
+    const mpm_ctx* c = batch->ctx[i];
+    args.push_back(make_sort_args(c->g, c->P[c->cur], c->P[1 - c->cur], (int)c->n, c->sb));
+    for (int k = 0; k < args[i].n_tiles; ++k) work.push_back(make_int2(i, k));
+  }
+  if (work.empty()) return MPM_OK;
+  sort_batch_args(args.data(), ns);
+  // (pageable sources: the copies have read them when the calls return)
+  BCU(cudaMemcpyAsync(batch->sort_d, args.data(), ns * sizeof(SortArgs), cudaMemcpyHostToDevice, s));
+  BCU(cudaMemcpyAsync(batch->sort_work_d, work.data(), work.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  launch_sort_batch(batch->sort_d, ns, args[0].passes, batch->sort_work_d, (int)work.size(), s);
   BCU(cudaGetLastError());
+  for (mpm_ctx* c : batch->ctx)
+    if (c->n > 0) c->cur = 1 - c->cur;
   return MPM_OK;
 }
 

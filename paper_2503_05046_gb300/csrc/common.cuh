@@ -35,7 +35,7 @@ struct GridDev {
   int rx, ry, rz;         // nodes per axis
   int nbx, nby, nbz;      // 4^3 blocks per axis
   int bc;                 // Dirichlet layers
-  int morton_bits;        // bits per axis of the block sort key
+  int morton_bits;        // bits of the block sort key on the longest axis
   int sort_cell_bits;     // 1: the sort key also orders cells within a block
   // Block-sparse storage (null: dense, every 4^3 block has its nodes at
   // block * 64): slot[b] is the storage block of grid block b during a
@@ -193,16 +193,6 @@ __device__ __forceinline__ long long storage_nodes(const GridDev& g) {
 // Active blocks that have storage (the pool caps a sparse grid's list).
 __device__ __forceinline__ int active_with_storage(const GridDev& g, int n_act) {
   return g.slot && n_act > g.pool_blocks ? g.pool_blocks : n_act;
-}
-
-__device__ __forceinline__ uint32_t spread_bits3(uint32_t v) {
-  // insert two zero bits between the low 10 bits of v
-  v &= 0x3ffu;
-  v = (v | (v << 16)) & 0x030000ffu;
-  v = (v | (v << 8)) & 0x0300f00fu;
-  v = (v | (v << 4)) & 0x030c30c3u;
-  v = (v | (v << 2)) & 0x09249249u;
-  return v;
 }
 
 // Quadratic B-spline stencil of the MLS-MPM transfers (free motion, Eq. (6)).

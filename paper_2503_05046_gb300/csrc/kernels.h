@@ -39,16 +39,37 @@ struct DevStats {
 struct SortBuffers {
   uint32_t* keys[2];
   uint32_t* vals[2];
-  uint32_t* hist;     // 256 * n_tiles
-  uint32_t* partial;  // scan partials
-  int hist_cap;
+  uint32_t* hist;     // sort_hist_len entries: digits x tiles, then the digits' totals
 };
 
+// One scene's sort, as its kernels take it.
+constexpr int kSortRoundsMin = 4, kSortRoundsMax = 8;
+struct SortArgs {
+  GridDev g;
+  Particles src, dst;
+  int n, n_tiles;
+  int rounds;         // rounds of 32 keys per warp of a tile (eight warps)
+  int bits, passes, digit;  // key bits, passes, bits per pass
+  uint32_t* keys[2];
+  uint32_t* vals[2];
+  uint32_t* hist;
+};
+
+int sort_key_bits(const GridDev& g);
+int sort_max_tiles(int n);
 int sort_hist_len(int n);
 cudaError_t sort_prepare();  // once per device: the small-scene sort's shared memory
-// ---- sort.cu: block keys, LSD radix sort (8-bit digits), permutation ----
+// ---- sort.cu: block keys, LSD radix sort, permutation ----
 void launch_sort(const GridDev& g, const Particles& src, const Particles& dst, int n,
                  SortBuffers& sb, cudaStream_t s);
+// batched: SortArgs per scene (device memory; sort_batch_args evens their passes
+// out), one (scene, tile) item per thread block; the sorted particles are in
+// each scene's dst
+SortArgs make_sort_args(const GridDev& g, const Particles& src, const Particles& dst, int n,
+                        const SortBuffers& sb);
+void sort_batch_args(SortArgs* args, int n_scenes);
+void launch_sort_batch(const SortArgs* args, int n_scenes, int passes, const int2* work, int n_work,
+                       cudaStream_t s);
 // gather particles of `src` into id order (out[pid] = state) for mem reads
 void launch_to_id_order(const Particles& P, int n, float* out_x, float* out_v, float* out_C,
                         float* out_F, cudaStream_t s);
