@@ -971,8 +971,8 @@ mpm_status mpm_set_particles(mpm_ctx* ctx, const float* x, const float* v, const
       dptr[f] = src[f];
     }
   }
-  launch_from_id_order(ctx->P[ctx->cur], (int)n, dptr[0], dptr[1], dptr[2], dptr[3], ctx->stream);
-  if (F) launch_stress_from_F(ctx->P[ctx->cur], (int)n, ctx->groups_d, ctx->stream);
+  launch_from_id_order(ctx->P[ctx->cur], (int)n, dptr[0], dptr[1], dptr[2], dptr[3],
+                       ctx->groups_d, ctx->stream);
   CU(cudaGetLastError());
   CU(cudaStreamSynchronize(ctx->stream));
   return MPM_OK;
@@ -1514,8 +1514,7 @@ namespace {
 // state buffer (24 floats per particle, id order) -> particle buffer `cur`
 void restore_state(mpm_ctx* ctx, const float* st, cudaStream_t s) {
   const size_t n = (size_t)ctx->n;
-  launch_from_id_order(ctx->P[ctx->cur], (int)n, st, st + 3 * n, st + 6 * n, st + 15 * n, s);
-  launch_stress_from_F(ctx->P[ctx->cur], (int)n, ctx->groups_d, s);
+  launch_from_id_order(ctx->P[ctx->cur], (int)n, st, st + 3 * n, st + 6 * n, st + 15 * n, ctx->groups_d, s);
 }
 
 void save_state(mpm_ctx* ctx, float* st, cudaStream_t s) {

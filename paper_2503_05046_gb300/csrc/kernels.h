@@ -74,7 +74,7 @@ void launch_sort_batch(const SortArgs* args, int n_scenes, int passes, const int
 void launch_to_id_order(const Particles& P, int n, float* out_x, float* out_v, float* out_C,
                         float* out_F, cudaStream_t s);
 void launch_from_id_order(const Particles& P, int n, const float* in_x, const float* in_v,
-                          const float* in_C, const float* in_F, cudaStream_t s);
+                          const float* in_C, const float* in_F, const DevGroup* groups, cudaStream_t s);
 // Kirchhoff stress planes from F (after F was set from outside)
 void launch_stress_from_F(const Particles& P, int n, const DevGroup* groups, cudaStream_t s);
 

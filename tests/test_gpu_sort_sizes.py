@@ -65,3 +65,26 @@ def test_batched_sort_keeps_every_particle():
                     assert np.array_equal(w[key], got[key]), key
     finally:
         batch.close()
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 257, 1000])
+@pytest.mark.parametrize("field", ["x", "v", "C", "F"])
+def test_one_field_set_and_read_in_id_order(n, field):
+    """Records of three and nine floats at the edges of a warp and of a block,
+    in an order that is not the ids': one field set, the others as they were,
+    and read with the others left out."""
+    from paper_2503_05046_gb300 import native
+    sim = native.Sim(scattered(n, (64, 64, 64)))
+    try:
+        want = give_state(sim, n)
+        sim.step(n_substeps=0)
+        want[field] = want[field] + np.float32(0.25)
+        native.mpm_set_particles(sim.ctx, **{{"C": "Cm"}.get(field, field): want[field]})
+        got = sim.get_particles()
+        for key in want:
+            assert np.array_equal(want[key], got[key]), key
+        one = np.empty_like(want[field])
+        native.mpm_get_particles(sim.ctx, **{{"C": "Cm"}.get(field, field): one})
+        assert np.array_equal(one, want[field])
+    finally:
+        sim.close()
