@@ -34,7 +34,7 @@ struct mpm_batch {
   long long n_all = 0;  // particles of all members, as the work lists have them
   int g2p_threads = 256;
   int grid_particles = 2048;
-  int solve_blocks = 1;  // blocks (one cluster) per scene's contact solve
+  int solve_blocks = 0;  // blocks (one cluster) per scene's contact solve; 0: by the scene count
   // per-scene argument records (device) and their host images
   P2GArgs* p2g_d = nullptr;
   GridBatchArgs* grid_d = nullptr;
@@ -195,6 +195,20 @@ std::vector<int2> build_work(mpm_batch* b) {
   return w;
 }
 
+// Blocks per scene's contact solve: as asked for, else by how many scenes share
+// the device, each line where the measured times cross (ms per step of four
+// substeps with 1, 2, 4 and 8 blocks; scenes of 2k particles up to the bound):
+//    24 scenes to 64k   4.27  2.65  1.99  1.71
+//    64 scenes to 32k   4.61  3.31  2.69  3.20
+//   128 scenes to 16k   4.04  3.18  2.79  3.59
+//   304 scenes to 8k    4.00  3.53  3.81  5.23
+//   400 scenes to 8k    4.71  4.51  5.00  6.70
+int solve_blocks_of(const mpm_batch* b) {
+  if (b->solve_blocks > 0) return b->solve_blocks;
+  const int ns = (int)b->ctx.size(), sms = b->ctx[0]->num_sms;
+  return 4 * ns <= sms ? 8 : ns <= sms ? 4 : ns <= 3 * sms ? 2 : 1;
+}
+
 cudaError_t enqueue(mpm_batch* b, int n_substeps, double dt) {
   const cudaStream_t s = b->stream;
   const int ns = (int)b->ctx.size();
@@ -202,7 +216,7 @@ cudaError_t enqueue(mpm_batch* b, int n_substeps, double dt) {
   for (int k = 0; k < n_substeps; ++k) {
     launch_p2g_batch(b->p2g_d, b->work_d, b->n_p2g, b->n_all, s);
     launch_grid_batch(b->grid_d, b->work_d + b->n_p2g, b->n_grid, s);
-    const cudaError_t e = launch_solve_batch(b->solve_d, b->order_d, ns, b->solve_blocks, s);
+    const cudaError_t e = launch_solve_batch(b->solve_d, b->order_d, ns, solve_blocks_of(b), s);
     if (e != cudaSuccess) return e;
     launch_g2p_batch(b->g2p_d, b->work_d + b->n_p2g + b->n_grid, b->n_g2p, b->g2p_threads, s);
   }
