@@ -195,6 +195,16 @@ __device__ __forceinline__ int active_with_storage(const GridDev& g, int n_act) 
   return g.slot && n_act > g.pool_blocks ? g.pool_blocks : n_act;
 }
 
+// First statement of every kernel launched by launch_chained: waits until the
+// kernel before it on the stream is complete and its writes are visible, then
+// lets the next one's blocks be set up beside this one's. (Their loads must not
+// pass the wait: what a kernel of the chain reads of an earlier one's is not
+// read through a const __restrict__ parameter, which the compiler may hoist.)
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Quadratic B-spline stencil of the MLS-MPM transfers (free motion, Eq. (6)).
 struct Stencil {
   int base[3];

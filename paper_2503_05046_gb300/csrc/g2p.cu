@@ -142,6 +142,7 @@ __device__ __forceinline__ void g2p_block(const G2PArgs& a, int block) {
 // kDense: a dense grid's node addresses (no block-table lookup)
 template <bool kDense>
 __global__ void __launch_bounds__(kThreads, 7) k_g2p(G2PArgs a) {
+  chain_begin();
   g2p_block<kDense>(a, blockIdx.x);
 }
 
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kThreads, 7) k_g2p(G2PArgs a) {
 __global__ void __launch_bounds__(512, 2) k_g2p_batch(const G2PArgs* __restrict__ args,
                                                       const int2* __restrict__ work) {
   __shared__ G2PArgs s_a;
+  chain_begin();
   const int2 wk = work[blockIdx.x];
   load_args(args + wk.x, s_a);
   __syncthreads();
@@ -160,14 +162,14 @@ __global__ void __launch_bounds__(512, 2) k_g2p_batch(const G2PArgs* __restrict_
 void launch_g2p(const G2PArgs& a, cudaStream_t s) {
   const int blocks = a.n > 0 ? (a.n + kThreads - 1) / kThreads : 1;
   if (a.g.slot)
-    k_g2p<false><<<blocks, kThreads, 0, s>>>(a);
+    launch_chained(k_g2p<false>, dim3(blocks), kThreads, 0, s, a);
   else
-    k_g2p<true><<<blocks, kThreads, 0, s>>>(a);
+    launch_chained(k_g2p<true>, dim3(blocks), kThreads, 0, s, a);
 }
 
 void launch_g2p_batch(const G2PArgs* args, const int2* work, int n_work, int threads,
                       cudaStream_t s) {
-  if (n_work > 0) k_g2p_batch<<<n_work, threads, 0, s>>>(args, work);
+  if (n_work > 0) launch_chained(k_g2p_batch, dim3(n_work), threads, 0, s, args, work);
 }
 
 }  // namespace mpmcr

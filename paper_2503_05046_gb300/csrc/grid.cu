@@ -49,9 +49,9 @@ __device__ __forceinline__ void compact_range(uint8_t* __restrict__ mark, int st
 // Sparse grids, before P2G: unmap the previous substep's blocks, then mark
 // the blocks of every particle's stencil (the nodes P2G, the solve and G2P
 // of this substep touch).
-__global__ void k_mark_sparse(GridDev g, Particles P, int n, uint8_t* __restrict__ mark,
-                              const int* __restrict__ act, const int* __restrict__ n_mapped,
-                              int* __restrict__ slot_tab) {
+__global__ void k_mark_sparse(GridDev g, Particles P, int n, uint8_t* mark, const int* act,
+                              const int* n_mapped, int* slot_tab) {
+  chain_begin();
   const int stride = gridDim.x * blockDim.x;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nm = *n_mapped;
@@ -71,6 +71,7 @@ __global__ void k_mark_sparse(GridDev g, Particles P, int n, uint8_t* __restrict
 __global__ void k_compact_sparse(uint8_t* __restrict__ mark, int n_blocks, int* __restrict__ act,
                                  int* __restrict__ n_act, int* __restrict__ slot_tab, int pool,
                                  uint32_t* __restrict__ status) {
+  chain_begin();
   compact_range(mark, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, n_blocks,
                 act, n_act, slot_tab, pool, status);
 }
@@ -149,6 +150,7 @@ __device__ __forceinline__ void grid_dense_range(const GridDev& g, const GridArr
 }
 
 __global__ void __launch_bounds__(256) k_grid_update_dense(GridDev g, GridArrays G, float h) {
+  chain_begin();
   grid_dense_range(g, G, h, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5),
                    (int)(gridDim.x * (blockDim.x >> 5)));
 }
@@ -170,6 +172,7 @@ __device__ __forceinline__ void grid_update_range(const GridDev& g, const GridAr
 }
 
 __global__ void __launch_bounds__(256) k_grid_update(GridDev g, GridArrays G, float h) {
+  chain_begin();
   grid_update_range(g, G, h, (long long)blockIdx.x * blockDim.x + threadIdx.x,
                     (long long)gridDim.x * blockDim.x, blockIdx.x == 0 && threadIdx.x == 0);
 }
@@ -179,6 +182,7 @@ __global__ void __launch_bounds__(256) k_grid_update(GridDev g, GridArrays G, fl
 __global__ void __launch_bounds__(256) k_grid_update_batch(const GridBatchArgs* __restrict__ args,
                                                            const int2* __restrict__ work) {
   __shared__ GridBatchArgs s_a;
+  chain_begin();
   const int2 wk = work[blockIdx.x];
   load_args(args + wk.x, s_a);
   __syncthreads();
@@ -191,30 +195,30 @@ __global__ void __launch_bounds__(256) k_grid_update_batch(const GridBatchArgs* 
 void launch_grid(const GridDev& g, const GridArrays& G, float h, int num_sms, cudaStream_t s) {
   const int n_blocks = g.nbx * g.nby * g.nbz;
   if (g.slot) {  // (compacted before P2G)
-    k_grid_update<<<num_sms * 8, 256, 0, s>>>(g, G, h);
+    launch_chained(k_grid_update, dim3(num_sms * 8), 256, 0, s, g, G, h);
     return;
   }
   // a warp per two blocks of the domain, up to eight thread blocks per SM
   int tb = (n_blocks + 15) / 16;
   tb = tb > num_sms * 8 ? num_sms * 8 : tb;
-  k_grid_update_dense<<<tb, 256, 0, s>>>(g, G, h);
+  launch_chained(k_grid_update_dense, dim3(tb), 256, 0, s, g, G, h);
 }
 
 void launch_sparse_map(const GridDev& g, const GridArrays& G, const Particles& P, int n,
                        int* slot_tab, uint32_t* status, int num_sms, cudaStream_t s) {
   const int n_blocks = g.nbx * g.nby * g.nbz;
   const int pb = (n + 255) / 256;
-  k_mark_sparse<<<pb < num_sms * 8 ? (pb > 0 ? pb : 1) : num_sms * 8, 256, 0, s>>>(
-      g, P, n, G.mark, G.act, G.n_mapped, slot_tab);
+  launch_chained(k_mark_sparse, dim3(pb < num_sms * 8 ? (pb > 0 ? pb : 1) : num_sms * 8), 256, 0, s, g, P,
+                 n, G.mark, G.act, G.n_mapped, slot_tab);
   int cb = (n_blocks + 255) / 256;
   cb = cb > num_sms * 8 ? num_sms * 8 : cb;
-  k_compact_sparse<<<cb, 256, 0, s>>>(G.mark, n_blocks, G.act, G.n_act, slot_tab, g.pool_blocks,
-                                      status);
+  launch_chained(k_compact_sparse, dim3(cb), 256, 0, s, G.mark, n_blocks, G.act, G.n_act, slot_tab,
+                 g.pool_blocks, status);
 }
 
 void launch_grid_batch(const GridBatchArgs* args, const int2* work, int n_work, cudaStream_t s) {
   if (n_work <= 0) return;
-  k_grid_update_batch<<<n_work, 256, 0, s>>>(args, work);
+  launch_chained(k_grid_update_batch, dim3(n_work), 256, 0, s, args, work);
 }
 
 }  // namespace mpmcr

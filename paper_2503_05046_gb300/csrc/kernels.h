@@ -9,6 +9,25 @@
 
 namespace mpmcr {
 
+// Launches a kernel that starts with chain_begin(): its blocks are set up while
+// the kernel before it drains, instead of after it. A substep is a chain of six
+// launches, several of which have a few microseconds of work or none.
+template <class... Params, class... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, int block, size_t smem, cudaStream_t s,
+                           Args... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 constexpr int kRedDoubles = 4 * 256 * 16;  // contact-solve partial sums: 4 slots x 256 blocks x 16
 // device-wide barrier of the cooperative solves: one 64-bit arrival counter
 // (words 0 and 1) on a line of its own

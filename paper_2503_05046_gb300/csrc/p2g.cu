@@ -409,6 +409,7 @@ __device__ __forceinline__ void p2g_walk_block(const P2GArgs& a, int block) {
 
 template <int ROUNDS, bool kDense>
 __global__ void __launch_bounds__(kWalkThreads, 24) k_p2g_w(P2GArgs a) {
+  chain_begin();
   p2g_walk_block<ROUNDS, kDense>(a, blockIdx.x);
 }
 
@@ -416,6 +417,7 @@ template <int ROUNDS>
 __global__ void __launch_bounds__(kWalkThreads, 24) k_p2g_w_batch(const P2GArgs* __restrict__ args,
                                                                  const int2* __restrict__ work) {
   __shared__ P2GArgs s_a;
+  chain_begin();
   const int2 wk = work[blockIdx.x];
   load_args(args + wk.x, s_a);
   __syncthreads();
@@ -430,9 +432,9 @@ void launch_walk(const P2GArgs& a, cudaStream_t s) {
   const int per_block = kWalkThreads * ROUNDS;
   const int nblk = (a.n + per_block - 1) / per_block;
   if (a.g.slot)
-    k_p2g_w<ROUNDS, false><<<nblk, kWalkThreads, walk_smem<ROUNDS>(), s>>>(a);
+    launch_chained(k_p2g_w<ROUNDS, false>, dim3(nblk), kWalkThreads, walk_smem<ROUNDS>(), s, a);
   else
-    k_p2g_w<ROUNDS, true><<<nblk, kWalkThreads, walk_smem<ROUNDS>(), s>>>(a);
+    launch_chained(k_p2g_w<ROUNDS, true>, dim3(nblk), kWalkThreads, walk_smem<ROUNDS>(), s, a);
 }
 
 template <class K>
@@ -464,9 +466,9 @@ int p2g_block_particles(long long n) { return kWalkThreads * (n < kWalkOneRound 
 void launch_p2g_batch(const P2GArgs* args, const int2* work, int n_work, long long n, cudaStream_t s) {
   if (n_work <= 0) return;
   if (n < kWalkOneRound)
-    k_p2g_w_batch<1><<<n_work, kWalkThreads, walk_smem<1>(), s>>>(args, work);
+    launch_chained(k_p2g_w_batch<1>, dim3(n_work), kWalkThreads, walk_smem<1>(), s, args, work);
   else
-    k_p2g_w_batch<3><<<n_work, kWalkThreads, walk_smem<3>(), s>>>(args, work);
+    launch_chained(k_p2g_w_batch<3>, dim3(n_work), kWalkThreads, walk_smem<3>(), s, args, work);
 }
 
 void launch_p2g(const P2GArgs& a, cudaStream_t s) {

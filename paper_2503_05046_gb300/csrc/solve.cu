@@ -1563,12 +1563,16 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) k_solve_small(SolveArgs a) { small_solve(a); }
+__global__ void __launch_bounds__(kThreads, 1) k_solve_small(SolveArgs a) {
+  chain_begin();
+  small_solve(a);
+}
 
 // Batched: a block per scene
 __global__ void __launch_bounds__(kThreads, 1) k_solve_small_batch(const SolveArgs* __restrict__ args,
                                                                    const int* __restrict__ order) {
   __shared__ SolveArgs s_a;
+  chain_begin();
   load_args(args + order[blockIdx.x], s_a);
   __syncthreads();
   if (threadIdx.x == 0) s_a.small_max = kSmallContacts;
@@ -1578,6 +1582,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve_small_batch(const SolveAr
 
 template <bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1) k_solve(SolveArgs a) {
+  chain_begin();
   solve_body<kCluster>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -1590,6 +1595,7 @@ template <int kBlocks>
 __global__ void __launch_bounds__(kThreads, 1) k_solve_batch(const SolveArgs* __restrict__ args,
                                                              const int* __restrict__ order) {
   __shared__ SolveArgs s_a;
+  chain_begin();
   load_args(args + order[blockIdx.x / kBlocks], s_a);
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -2403,26 +2409,29 @@ cudaError_t solve_prepare() {
 }
 
 namespace {
-cudaLaunchConfig_t cluster_config(int blocks, cudaLaunchAttribute* attr, cudaStream_t s) {
+// a cluster of `blocks`, chained as launch_chained's kernels are
+cudaLaunchConfig_t cluster_config(int blocks, cudaLaunchAttribute (&attr)[2], cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = solve_dynamic_smem();
   cfg.stream = s;
-  attr->id = cudaLaunchAttributeClusterDimension;
-  attr->val.clusterDim.x = blocks;
-  attr->val.clusterDim.y = 1;
-  attr->val.clusterDim.z = 1;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = blocks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cfg;
 }
 }  // namespace
 
 int solve_cluster_blocks() {
   for (int blocks : {16, 8, 4}) {
-    cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = cluster_config(blocks, &attr, nullptr);
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(blocks, attr, nullptr);
     int clusters = 0;
     if (cudaOccupancyMaxActiveClusters(&clusters, reinterpret_cast<const void*>(&k_solve<true>),
                                        &cfg) == cudaSuccess &&
@@ -2437,9 +2446,9 @@ cudaError_t launch_solve(const SolveArgs& a, int grid_blocks, int cluster_blocks
   SolveArgs args = a;
   if (cluster_blocks > 0 && args.cluster_max > 0) {
     args.small_max = args.cluster_max < kSmallContacts ? args.cluster_max : kSmallContacts;
-    k_solve_small<<<1, kThreads, kSmallSmem, s>>>(args);
-    cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = cluster_config(cluster_blocks, &attr, s);
+    launch_chained(k_solve_small, dim3(1), kThreads, kSmallSmem, s, args);
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(cluster_blocks, attr, s);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k_solve<true>, args);
     if (e != cudaSuccess) return e;
   } else {
@@ -2457,14 +2466,11 @@ template <int kBlocks>
 cudaError_t launch_solve_batch_k(const SolveArgs* args, const int* order, int n_scenes,
                                  cudaStream_t s) {
   if (kBlocks == 1) {
-    k_solve_batch<1><<<n_scenes, kThreads, solve_dynamic_smem(), s>>>(args, order);
-    return cudaGetLastError();
+    return launch_chained(k_solve_batch<1>, dim3(n_scenes), kThreads, solve_dynamic_smem(), s, args, order);
   }
-  cudaLaunchAttribute attr;
-  const cudaLaunchConfig_t cfg0 = cluster_config(kBlocks, &attr, s);
-  cudaLaunchConfig_t cfg = cfg0;
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = cluster_config(kBlocks, attr, s);
   cfg.gridDim = dim3(n_scenes * kBlocks);
-  cfg.attrs = &attr;
   return cudaLaunchKernelEx(&cfg, k_solve_batch<kBlocks>, args, order);
 }
 }  // namespace
@@ -2472,7 +2478,7 @@ cudaError_t launch_solve_batch_k(const SolveArgs* args, const int* order, int n_
 cudaError_t launch_solve_batch(const SolveArgs* args, const int* order, int n_scenes,
                                int blocks_per_scene, cudaStream_t s) {
   if (n_scenes <= 0) return cudaSuccess;
-  k_solve_small_batch<<<n_scenes, kThreads, kSmallSmem, s>>>(args, order);
+  launch_chained(k_solve_small_batch, dim3(n_scenes), kThreads, kSmallSmem, s, args, order);
   switch (blocks_per_scene) {
     case 2: return launch_solve_batch_k<2>(args, order, n_scenes, s);
     case 4: return launch_solve_batch_k<4>(args, order, n_scenes, s);

@@ -174,7 +174,10 @@ __device__ __forceinline__ void sort_small(const SortArgs& a) {
   for (int i = tid; i < a.n; i += kSmallSortThreads) a.vals[0][i] = idx_in[i];
 }
 
-__global__ void __launch_bounds__(kSmallSortThreads) k_sort_small(SortArgs a) { sort_small(a); }
+__global__ void __launch_bounds__(kSmallSortThreads) k_sort_small(SortArgs a) {
+  chain_begin();
+  sort_small(a);
+}
 
 // Histogram of digit `pass` over tile `tile` (a.rounds x 32 keys per warp); the
 // first pass forms the keys.
@@ -317,9 +320,16 @@ __device__ __forceinline__ void sort_scatter(const SortArgs& a, int pass, int ti
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_sort_hist(SortArgs a, int pass) { sort_hist(a, pass, blockIdx.x); }
-__global__ void __launch_bounds__(kThreads) k_sort_rows(SortArgs a) { sort_rows(a, blockIdx.x); }
+__global__ void __launch_bounds__(kThreads) k_sort_hist(SortArgs a, int pass) {
+  chain_begin();
+  sort_hist(a, pass, blockIdx.x);
+}
+__global__ void __launch_bounds__(kThreads) k_sort_rows(SortArgs a) {
+  chain_begin();
+  sort_rows(a, blockIdx.x);
+}
 __global__ void __launch_bounds__(kThreads) k_sort_scatter(SortArgs a, int pass) {
+  chain_begin();
   sort_scatter(a, pass, blockIdx.x);
 }
 
@@ -329,6 +339,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_scatter(SortArgs a, int pass)
 __global__ void __launch_bounds__(kThreads) k_sort_hist_batch(const SortArgs* __restrict__ args,
                                                               const int2* __restrict__ work, int pass) {
   __shared__ SortArgs s_a;
+  chain_begin();
   const int2 wk = work[blockIdx.x];
   load_args(args + wk.x, s_a);
   __syncthreads();
@@ -336,6 +347,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_hist_batch(const SortArgs* __
 }
 __global__ void __launch_bounds__(kThreads) k_sort_rows_batch(const SortArgs* __restrict__ args) {
   __shared__ SortArgs s_a;
+  chain_begin();
   load_args(args + blockIdx.x, s_a);
   __syncthreads();
   if (s_a.n > 0) sort_rows(s_a, blockIdx.y);
@@ -343,6 +355,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_rows_batch(const SortArgs* __
 __global__ void __launch_bounds__(kThreads) k_sort_scatter_batch(const SortArgs* __restrict__ args,
                                                                  const int2* __restrict__ work, int pass) {
   __shared__ SortArgs s_a;
+  chain_begin();
   const int2 wk = work[blockIdx.x];
   load_args(args + wk.x, s_a);
   __syncthreads();
@@ -350,7 +363,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_scatter_batch(const SortArgs*
 }
 
 __device__ __forceinline__ void permute_one(const Particles& src, const Particles& dst,
-                                            const uint32_t* __restrict__ perm, int i) {
+                                            const uint32_t* perm, int i) {
   // every plane's load before the first store: the compiler may not move a
   // load of src above a store to dst
   const uint32_t j = perm[i];
@@ -365,7 +378,8 @@ __device__ __forceinline__ void permute_one(const Particles& src, const Particle
   dst.grp[i] = grp;
 }
 
-__global__ void k_permute(Particles src, Particles dst, const uint32_t* __restrict__ perm, int n) {
+__global__ void k_permute(Particles src, Particles dst, const uint32_t* perm, int n) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) permute_one(src, dst, perm, i);
 }
@@ -373,6 +387,7 @@ __global__ void k_permute(Particles src, Particles dst, const uint32_t* __restri
 __global__ void __launch_bounds__(kThreads) k_permute_batch(const SortArgs* __restrict__ args,
                                                             const int2* __restrict__ work) {
   __shared__ SortArgs s_a;
+  chain_begin();
   const int2 wk = work[blockIdx.x];
   load_args(args + wk.x, s_a);
   __syncthreads();
@@ -556,16 +571,16 @@ void launch_sort(const GridDev& g, const Particles& src, const Particles& dst, i
   const SortArgs a = sort_args(g, src, dst, n, sb);
   int out = 0;
   if (n <= kSmallSortMax) {
-    k_sort_small<<<1, kSmallSortThreads, kSmallSortSmem, s>>>(a);
+    launch_chained(k_sort_small, dim3(1), kSmallSortThreads, kSmallSortSmem, s, a);
   } else {
     for (int p = 0; p < a.passes; ++p) {
-      k_sort_hist<<<a.n_tiles, kThreads, 0, s>>>(a, p);
-      k_sort_rows<<<1 << a.digit, kThreads, 0, s>>>(a);
-      k_sort_scatter<<<a.n_tiles, kThreads, 0, s>>>(a, p);
+      launch_chained(k_sort_hist, dim3(a.n_tiles), kThreads, 0, s, a, p);
+      launch_chained(k_sort_rows, dim3(1 << a.digit), kThreads, 0, s, a);
+      launch_chained(k_sort_scatter, dim3(a.n_tiles), kThreads, 0, s, a, p);
     }
     out = a.passes & 1;
   }
-  k_permute<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(src, dst, sb.vals[out], n);
+  launch_chained(k_permute, dim3((n + kThreads - 1) / kThreads), kThreads, 0, s, src, dst, sb.vals[out], n);
 }
 
 // a batch's scenes: every one takes the passes of the one with the most
@@ -588,11 +603,11 @@ void launch_sort_batch(const SortArgs* args, int n_scenes, int passes, const int
                        cudaStream_t s) {
   if (n_work <= 0) return;
   for (int p = 0; p < passes; ++p) {
-    k_sort_hist_batch<<<n_work, kThreads, 0, s>>>(args, work, p);
-    k_sort_rows_batch<<<dim3(n_scenes, kMaxBins), kThreads, 0, s>>>(args);
-    k_sort_scatter_batch<<<n_work, kThreads, 0, s>>>(args, work, p);
+    launch_chained(k_sort_hist_batch, dim3(n_work), kThreads, 0, s, args, work, p);
+    launch_chained(k_sort_rows_batch, dim3(n_scenes, kMaxBins), kThreads, 0, s, args);
+    launch_chained(k_sort_scatter_batch, dim3(n_work), kThreads, 0, s, args, work, p);
   }
-  k_permute_batch<<<n_work, kThreads, 0, s>>>(args, work);
+  launch_chained(k_permute_batch, dim3(n_work), kThreads, 0, s, args, work);
 }
 
 void launch_to_id_order(const Particles& P, int n, float* ox, float* ov, float* oC, float* oF,
