@@ -517,7 +517,7 @@ mpm_status mpm_synchronize(mpm_ctx* ctx);
    solved by one thread-block cluster (up to 16 SMs exchanging their sums
    through distributed shared memory, hardware cluster barriers); more
    contacts go to the cooperative launch over as many SMs as they need, with
-   device-wide barriers (default 4096; 0: always the cooperative launch).
+   device-wide barriers (default 1024; 0: always the cooperative launch).
    MPM_OPT_CLUSTER_BLOCKS: thread blocks (SMs) in that cluster, a power of two
    up to the largest the device schedules (0, the default: the largest, 16 on
    GB300).

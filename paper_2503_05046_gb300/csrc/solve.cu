@@ -24,16 +24,26 @@
 //      is monotone (f convex); each pass evaluates it at 8 points in one
 //      contact sweep: first on a geometric grid (0, 4^-5 .. 4) to bracket the
 //      root, then at the Newton and secant estimates and points that split
-//      the bracket, until |f'| <= ls_rel_tol |f'(0)|. Up to kLocalLsMax contacts every block
-//      runs the whole line search by itself over all contacts (their v_c and
-//      dv_c sit in L2), so its passes need no grid barrier; above that the
-//      contacts are split over the blocks and each pass ends in a grid-wide
+//      the bracket, until |f'| <= ls_rel_tol |f'(0)|. Up to kLocalLsMax
+//      contacts every block runs the whole line search by itself over all
+//      contacts (their v_c and dv_c sit in L2), so its passes need no grid
+//      barrier; above that each block takes the contacts whose dv_c it formed
+//      in phase C (no barrier between the two) and each pass ends in a grid-wide
 //      reduction.
 // Every block reads the same reduced sums (or computes the same ones in the
 // same order), so all take the same decisions. Scalar sums are accumulated
 // per thread and per warp in FP32, across warps and blocks as double-float
 // (hi, lo) pairs with error-free FP32 transforms: GB300's FP64 pipe is narrow
 // enough that FP64 on these serial paths costs more than the rest of a pass.
+//
+// Bound by latency: barriers (a pass of the line search, 4.5 us with 40,000
+// contacts, is nearly all barrier) and the L2 round trips between them; phase G
+// by its reductions. Per iteration of the manipulation scene (40,080 contacts,
+// 38,355 contact nodes): G 20.3 -> 12.3 us (node sums kept over runs of contacts
+// in a cell, gathers through L1), N 12.8 -> 5.9 (a node's loads issued together),
+// C and the line search 19.7 -> 16.6 (no barrier after C). The scoop's ten
+// substeps (3,105 contacts): 1,303 -> 706 us, of which the cooperative launch in
+// place of the cluster is 580.
 #include <cfloat>
 
 #include "kernels.h"
@@ -44,9 +54,14 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr int kContactsPerBlock = 128;  // forward solve: 8 contacts per warp in the gather phases
+// Contacts per block of the cooperative launch: as few as spread a solve over the
+// device, the phases being bound by each SM's reductions and loads (3,105
+// contacts, 56,000 contact nodes, one step of ten substeps: 1,099 us with 128,
+// 902 with 64, 823 with 32, 777 with 16; below, a warp's lanes would be idle).
+constexpr int kContactsPerBlock = 16;
 constexpr int kAdjContactsPerBlock = 16;  // adjoint: one contact per warp
-constexpr int kLocalLsMax = 4096;      // up to this many contacts each block line-searches alone
+// Up to this many contacts (one per thread) each block line-searches alone.
+constexpr int kLocalLsMax = kThreads;
 constexpr int kLsPoints = 8;
 constexpr int kRedWidth = 16;              // (hi, lo) pairs per block and reduction
 constexpr int kMaxSolveBlocks = 256;
@@ -304,6 +319,7 @@ __device__ __forceinline__ LaneNode lane_node(const GridDev& g, const float4& xp
 constexpr int kGrp = 4;
 constexpr int kGrpPerWarp = 32 / kGrp;
 constexpr int kGrpNodes = (27 + kGrp - 1) / kGrp;
+constexpr int kRoundContacts = kWarps * kGrpPerWarp;  // a block's contacts per round
 
 struct GroupNodes {
   int node[kGrpNodes];
@@ -323,6 +339,19 @@ __device__ __forceinline__ void group_nodes(const GridDev& g, const float4& xp, 
     r.w[j] = c < 27 ? s.w[0][cx] * s.w[1][cy] * s.w[2][cz] : 0.f;
   }
 }
+
+// B-spline weight of node offset o in {0, 1, 2} at fraction f as a + b t^2 with
+// t = s f + k: the same roundings as stencil()'s, with the lane's coefficients.
+struct NodeWeight {
+  float s, k, b, a;
+  __device__ __forceinline__ explicit NodeWeight(int o)
+      : s(o == 0 ? -1.f : 1.f), k(o == 0 ? 1.5f : o == 1 ? -1.f : -0.5f), b(o == 1 ? -1.f : 0.5f),
+        a(o == 1 ? 0.75f : 0.f) {}
+  __device__ __forceinline__ float at(float f) const {
+    const float t = fmaf(s, f, k);
+    return fmaf(b * t, t, a);
+  }
+};
 
 // compensated sum of (S, E) pairs over the lanes of a group, bitwise the same
 // in each of them (TwoSum's error term is exact whichever operand comes first)
@@ -357,7 +386,7 @@ __device__ __forceinline__ void load_contact(const Contacts& C, int p, float4& x
 // line form in shared-memory slot k * kThreads + tid across the passes of one
 // line search, packed into three float4: (v_n, e_n, vhat, phi0),
 // (mu n0, body, v_t.x, v_t.y), (v_t.z, e_t); k and d come from the body table.
-constexpr int kLsCacheDepth = 4;
+constexpr int kLsCacheDepth = 2;  // (four took the L1 more than it saved)
 constexpr int kLsCacheSlots = kLsCacheDepth * kThreads;
 
 __device__ __forceinline__ void line_store(float4* cache, int slot, const ContactLine& L, int body) {
@@ -1130,6 +1159,9 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   __shared__ float2 s_A, s_B;
   __shared__ float s_alpha;
   __shared__ int s_dec;
+  // phase G, per warp and contact: gradient and H00; H11, H22, H01, H02; H12 and
+  // the fractions; the base node
+  __shared__ float4 s_con[kWarps][kGrpPerWarp][4];
   extern __shared__ float4 s_line[];  // 3 x kLsCacheSlots: the line-search cache (+ stencils)
   LineSearch ls;  // used by warp 0
   const int tid = threadIdx.x;
@@ -1152,8 +1184,9 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   for (int i = tid; i < kMaxBodies * 6; i += kThreads) (&s_imp[0][0])[i] = 0.f;
   __syncthreads();
 
-  // phase timers (block 0, thread 0): list, G, N, line search, impulses
-  PhaseClock clk;
+  // phase timers (block 0, thread 0): list, G, N, line search, impulses (in
+  // shared memory: sixteen registers of every thread otherwise)
+  __shared__ PhaseClock clk;
   if (block == 0 && tid == 0) clk.start();
   auto lap = [&](int ph) {
     if (block == 0 && tid == 0) clk.lap(ph);
@@ -1162,11 +1195,16 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   // barrier then waits for arrivals that never come)
   Barrier B{a.bar, (unsigned)nblk, a.status, a.poison, kCluster ? 1 : 0,
             kCluster ? 0u : (unsigned)a.wait_extra, (unsigned)block};
-  const int gtid = block * kThreads + tid;
-  const int gstride = nblk * kThreads;
+  // Warps are numbered across the blocks, not block by block: a phase whose items
+  // don't fill every warp (or every warp's last round) then has them on as many
+  // SMs as there are, which the reductions of phase G (one per clock and SM)
+  // and the atomics of the list are bound by. Block by block, 402 contacts sat on
+  // four of the sixteen blocks.
   const int lane = tid & 31;
-  const int gwarp = gtid >> 5;
-  const int nwarps = gstride >> 5;
+  const int gwarp = (tid >> 5) * nblk + block;
+  const int nwarps = nblk * kWarps;
+  const int gtid = gwarp * 32 + lane;
+  const int gstride = nblk * kThreads;
   const GridDev& g = a.g;
   // per-block partial sums, a ring of 4 slots of kMaxSolveBlocks x kRedWidth;
   // a slot is rewritten two reductions later, after every block has read it
@@ -1195,21 +1233,32 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
     if (gtid == 0) *a.poison = 0;
   }
 
-  // ---- contact-node list: the union of the contacts' stencils (a thread
-  // per contact; the warp takes its list slots with one atomic)
-  for (int p0 = gtid & ~31; p0 < nc; p0 += gstride) {
-    const int p = p0 + lane;
-    int node[27];
-    unsigned won = 0u;  // 27 bits: this thread claimed the node first
-    if (p < nc) {
-      const float4 xp = a.C.xp[p];
-      Stencil s;
-      stencil(g, xp.x, xp.y, xp.z, s);
+  // Phases that go over stencils: kGrp lanes per contact (lane group grp of the
+  // warp, lane sub of the group owns stencil nodes sub, sub + kGrp, ...), so
+  // a warp works on kGrpPerWarp contacts at once. The stencils of a warp's
+  // first round stay in shared memory across the iterations, beside the
+  // line-search cache (registers are kept for the gathers in flight).
+  const int grp = lane / kGrp, sub = lane % kGrp;
+  const int wfirst = gwarp * kGrpPerWarp;
+  const int rstride = nwarps * kGrpPerWarp;
+  int* s_own_node = reinterpret_cast<int*>(s_line + 3 * kLsCacheSlots) + tid * kGrpNodes;
+  float* s_own_w = reinterpret_cast<float*>(s_line + 3 * kLsCacheSlots) + kThreads * kGrpNodes +
+                   tid * kGrpNodes;
+
+  // ---- contact-node list: the union of the contacts' stencils (the warp takes
+  // its list slots with one atomic)
+  for (int base = wfirst; base < nc; base += rstride) {
+    const int p = base + grp;
+    GroupNodes gn;
+    group_nodes(g, p < nc ? a.C.xp[p] : make_float4(0.f, 0.f, 0.f, 0.f), sub, gn);
+    unsigned won = 0u;  // kGrpNodes bits: this thread claimed the node first
 #pragma unroll
-      for (int c = 0; c < 27; ++c) {
-        node[c] = node_index(g, s.base[0] + c % 3, s.base[1] + (c / 3) % 3, s.base[2] + c / 9);
-        if (atomicExch(a.G.cflag + node[c], 1) == 0) won |= 1u << c;
+    for (int j = 0; j < kGrpNodes; ++j) {
+      if (base == wfirst) {
+        s_own_node[j] = gn.node[j];
+        s_own_w[j] = gn.w[j];
       }
+      if (p < nc && sub + kGrp * j < 27 && atomicExch(a.G.cflag + gn.node[j], 1) == 0) won |= 1u << j;
     }
     const int cnt = __popc(won);
     int incl = cnt;  // inclusive prefix sum over the warp
@@ -1221,14 +1270,12 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
     int slot0 = 0;
     if (lane == 31 && incl > 0) slot0 = atomicAdd(a.G.n_cnodes, incl);
     int slot = __shfl_sync(0xffffffffu, slot0, 31) + incl - cnt;
-    if (won) {
 #pragma unroll
-      for (int c = 0; c < 27; ++c)
-        if ((won >> c) & 1u) {
-          if (slot < a.G.cnodes_cap) a.G.cnodes[slot] = node[c];
-          ++slot;
-        }
-    }
+    for (int j = 0; j < kGrpNodes; ++j)
+      if ((won >> j) & 1u) {
+        if (slot < a.G.cnodes_cap) a.G.cnodes[slot] = gn.node[j];
+        ++slot;
+      }
   }
   if (!grid_sync(B)) return;
   lap(0);
@@ -1248,29 +1295,6 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   float4* vnxt = a.G.v2;
   float4* lcur = a.G.vlo;
   float4* lnxt = a.G.vlo2;
-  // Gather / scatter phases: kGrp lanes per contact (lane group grp of the
-  // warp, lane sub of the group owns stencil nodes sub, sub + kGrp, ...), so
-  // a warp works on kGrpPerWarp contacts at once. The contacts of a warp's
-  // first round stay in registers across the iterations.
-  const int grp = lane / kGrp, sub = lane % kGrp;
-  const int wfirst = gwarp * kGrpPerWarp;
-  const int rstride = nwarps * kGrpPerWarp;
-  const int own_p = wfirst + grp;
-  const bool own = own_p < nc;
-  // (the stencil of that contact in shared memory, beside the line-search
-  // cache: registers are kept for the gathers in flight)
-  int* s_own_node = reinterpret_cast<int*>(s_line + 3 * kLsCacheSlots) + tid * kGrpNodes;
-  float* s_own_w = reinterpret_cast<float*>(s_line + 3 * kLsCacheSlots) + kThreads * kGrpNodes +
-                   tid * kGrpNodes;
-  {
-    GroupNodes gn;
-    group_nodes(g, own ? a.C.xp[own_p] : make_float4(0.f, 0.f, 0.f, 0.f), sub, gn);
-#pragma unroll
-    for (int j = 0; j < kGrpNodes; ++j) {
-      s_own_node[j] = gn.node[j];
-      s_own_w[j] = gn.w[j];
-    }
-  }
   auto own_nodes = [&](GroupNodes& gn) {
 #pragma unroll
     for (int j = 0; j < kGrpNodes; ++j) {
@@ -1281,8 +1305,10 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   // this thread's first contact node (the list is fixed for the solve)
   const int my_node = gtid < ncn ? a.G.cnodes[gtid] : -1;
   // line search alone in each block (no grid barrier) or split over blocks
-  const bool local_ls = kCluster ? nc <= kThreads : nc <= kLocalLsMax;
-  const int ls_first = local_ls ? tid : gtid, ls_stride = local_ls ? kThreads : gstride;
+  const bool local_ls = nc <= kLocalLsMax;
+  // (split, a block takes the contacts that its own warps take in phase C, so
+  // that no grid barrier comes between the two)
+  const int ls_items = local_ls ? nc : (nc + rstride - 1) / rstride * kRoundContacts;
   Barrier Bl{nullptr, 1u, a.status, nullptr, 0, 0u, 0u};
   const float eps2 = a.eps_s * a.eps_s;
   float alpha = 0.f;
@@ -1306,8 +1332,8 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
 #pragma unroll
           for (int j = 0; j < kGrpNodes; ++j) {
             if (sub + kGrp * j >= 27) continue;
-            hq[j] = __ldcg(vcur + gn.node[j]);
-            lq[j] = __ldcg(lcur + gn.node[j]);
+            hq[j] = vcur[gn.node[j]];
+            lq[j] = lcur[gn.node[j]];
           }
 #pragma unroll
           for (int j = 0; j < kGrpNodes; ++j) {
@@ -1349,13 +1375,17 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
       float gr[3], H[6];
       contact_grad(L, n, gr);
       contact_hess(L, n, H);
-#pragma unroll
-      for (int j = 0; j < kGrpNodes; ++j) {
-        if (sub + kGrp * j >= 27) continue;
-        const float w = gn.w[j], w2 = w * w;
-        red_add_v4(a.G.acc0 + gn.node[j], w * gr[0], w * gr[1], w * gr[2], w2 * H[0]);
-        red_add_v4(a.G.acc1 + gn.node[j], w2 * H[1], w2 * H[2], w2 * H[3], w2 * H[4]);
-        red_add_f32(a.G.acc2 + gn.node[j], w2 * H[5]);
+      float4* rec = s_con[tid >> 5][grp];
+      if (sub == 0) {
+        rec[0] = make_float4(gr[0], gr[1], gr[2], H[0]);
+      } else if (sub == 1) {
+        rec[1] = make_float4(H[1], H[2], H[3], H[4]);
+      } else {
+        Stencil st;
+        stencil(g, xp.x, xp.y, xp.z, st);
+        rec[sub] = sub == 2 ? make_float4(H[5], st.fx[0], st.fx[1], st.fx[2])
+                            : make_float4(__int_as_float(st.base[0]), __int_as_float(st.base[1]),
+                                          __int_as_float(st.base[2]), 0.f);
       }
     };
     for (int base = wfirst; base < nc; base += rstride) {
@@ -1376,6 +1406,50 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
         group_nodes(g, xp, sub, gn);
       const float n3[3] = {q.x, q.y, q.z};
       phase_g(p, valid, xp, n3, q.w, bb, body, gn);
+      __syncwarp();
+      // Node sums: a lane per stencil node goes over the warp's contacts and
+      // keeps its sums while the base node stays the same. Neighbouring contacts
+      // mostly share a cell (P2G registers them in the particles' order): three
+      // runs per eight contacts at 4 to 8 particles per cell, so a third of the
+      // reductions, which is what bounds the phase (0.9 per clock and SM).
+      if (lane < 27) {
+        const int cx = lane % 3, cy = lane / 3 % 3, cz = lane / 9;
+        const NodeWeight wx(cx), wy(cy), wz(cz);
+        const int m = min(kGrpPerWarp, nc - base);
+        int node = -1, b0 = 0, b1 = 0, b2 = 0;
+        float t[9];
+        auto flush = [&]() {
+          red_add_v4(a.G.acc0 + node, t[0], t[1], t[2], t[3]);
+          red_add_v4(a.G.acc1 + node, t[4], t[5], t[6], t[7]);
+          red_add_f32(a.G.acc2 + node, t[8]);
+        };
+        for (int k = 0; k < m; ++k) {
+          const float4* rec = s_con[tid >> 5][k];
+          const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
+          const int n0 = __float_as_int(r3.x), n1 = __float_as_int(r3.y), n2 = __float_as_int(r3.z);
+          if (node < 0 || n0 != b0 || n1 != b1 || n2 != b2) {
+            if (node >= 0) flush();
+            b0 = n0;
+            b1 = n1;
+            b2 = n2;
+            node = node_index(g, b0 + cx, b1 + cy, b2 + cz);
+#pragma unroll
+            for (int c = 0; c < 9; ++c) t[c] = 0.f;
+          }
+          const float w = wx.at(r2.y) * wy.at(r2.z) * wz.at(r2.w), w2 = w * w;
+          t[0] = fmaf(w, r0.x, t[0]);
+          t[1] = fmaf(w, r0.y, t[1]);
+          t[2] = fmaf(w, r0.z, t[2]);
+          t[3] = fmaf(w2, r0.w, t[3]);
+          t[4] = fmaf(w2, r1.x, t[4]);
+          t[5] = fmaf(w2, r1.y, t[5]);
+          t[6] = fmaf(w2, r1.z, t[6]);
+          t[7] = fmaf(w2, r1.w, t[7]);
+          t[8] = fmaf(w2, r2.x, t[8]);
+        }
+        flush();
+      }
+      __syncwarp();
     }
     if (!grid_sync(B)) return;
     lap(1);
@@ -1386,34 +1460,47 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
     float2* slot = next_slot();
     {
       float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // G2, P2 - P*2, J2, A, B
+      // (a node's loads go out while the one before it is worked on: with the
+      // list entry, the node and the step one after the other, a round of a
+      // thread took 6.5 us)
+      struct NodeIn {
+        float4 vs, v, vl, d, c0, c1;
+        float c2;
+      } in;
+      auto fetch = [&](int node) {
+        in.vs = a.G.vs[node];
+        in.v = vcur[node];
+        in.vl = lcur[node];
+        in.d = it > 0 ? a.G.dv[node] : make_float4(0.f, 0.f, 0.f, 0.f);
+        // written by other blocks' reductions in this launch: read from L2
+        in.c0 = __ldcg(a.G.acc0 + node);
+        in.c1 = __ldcg(a.G.acc1 + node);
+        in.c2 = __ldcg(a.G.acc2 + node);
+      };
+      int next = my_node;
       for (int t = gtid; t < ncn; t += gstride) {
-        const int node = t == gtid ? my_node : a.G.cnodes[t];
-        const float4 vs = a.G.vs[node];
-        const float m = vs.w;
-        float4 v = vcur[node];
-        float4 vl = lcur[node];
+        const int cur = next;
+        fetch(cur);
+        if (t + gstride < ncn) next = a.G.cnodes[t + gstride];
+        const NodeIn& q = in;
+        float4 v = q.v, vl = q.vl;
         if (it > 0) {
-          const float4 d = a.G.dv[node];
-          dd_add(v.x, vl.x, al * d.x);
-          dd_add(v.y, vl.y, al * d.y);
-          dd_add(v.z, vl.z, al * d.z);
-          vnxt[node] = v;
-          lnxt[node] = vl;
+          dd_add(v.x, vl.x, al * q.d.x);
+          dd_add(v.y, vl.y, al * q.d.y);
+          dd_add(v.z, vl.z, al * q.d.z);
+          vnxt[cur] = v;
+          lnxt[cur] = vl;
         }
         float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
-        // written by other blocks' reductions in this launch: read from L2
-        const float4 c0 = __ldcg(a.G.acc0 + node);
-        const float4 c1 = __ldcg(a.G.acc1 + node);
-        const float c2 = __ldcg(a.G.acc2 + node);
-        a.G.acc0[node] = make_float4(0.f, 0.f, 0.f, 0.f);
-        a.G.acc1[node] = make_float4(0.f, 0.f, 0.f, 0.f);
-        a.G.acc2[node] = 0.f;
-        if (m > 0.f && v.w == 0.f) {  // free DoF (v.w flags a Dirichlet node)
+        a.G.acc0[cur] = make_float4(0.f, 0.f, 0.f, 0.f);
+        a.G.acc1[cur] = make_float4(0.f, 0.f, 0.f, 0.f);
+        a.G.acc2[cur] = 0.f;
+        if (q.vs.w > 0.f && v.w == 0.f) {  // free DoF (v.w flags a Dirichlet node)
           // v - v* with the low part of the iterate
-          const float r0 = (v.x - vs.x) + vl.x, r1 = (v.y - vs.y) + vl.y, r2 = (v.z - vs.z) + vl.z;
-          node_step(m, vs, r0, r1, r2, c0, c1, c2, dv.x, dv.y, dv.z, acc);
+          const float r0 = (v.x - q.vs.x) + vl.x, r1 = (v.y - q.vs.y) + vl.y, r2 = (v.z - q.vs.z) + vl.z;
+          node_step(q.vs.w, q.vs, r0, r1, r2, q.c0, q.c1, q.c2, dv.x, dv.y, dv.z, acc);
         }
-        a.G.dv[node] = dv;
+        a.G.dv[cur] = dv;
       }
       if (it > 0) {
         float4* t = vcur; vcur = vnxt; vnxt = t;
@@ -1452,7 +1539,7 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
         float4 dq[kGrpNodes];
 #pragma unroll
         for (int j = 0; j < kGrpNodes; ++j)
-          if (sub + kGrp * j < 27) dq[j] = __ldcg(a.G.dv + gn.node[j]);
+          if (sub + kGrp * j < 27) dq[j] = a.G.dv[gn.node[j]];
 #pragma unroll
         for (int j = 0; j < kGrpNodes; ++j) {
           if (sub + kGrp * j >= 27) continue;
@@ -1467,7 +1554,11 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
         for (int o = 1; o < kGrp; o <<= 1) e[c] += __shfl_xor_sync(0xffffffffu, e[c], o);
       if (valid && sub == 0) a.C.dvc[p] = make_float4(e[0], e[1], e[2], 0.f);
     }
-    if (!grid_sync(B)) return;
+    if (local_ls) {
+      if (!grid_sync(B)) return;
+    } else {
+      __syncthreads();
+    }
     // ---- L: line-search passes of 8 points each (thread per contact)
     for (int pass = 0;; ++pass) {
       float2* sl = local_ls ? nullptr : next_slot();
@@ -1478,7 +1569,12 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
 #pragma unroll
       for (int k = 0; k < 2 * kLsPoints; ++k) acc[k] = 0.f;
       int k = 0;
-      for (int p = ls_first; p < nc; p += ls_stride, ++k) {
+      for (int i = tid; i < ls_items; i += kThreads, ++k) {
+        const int q = i % kRoundContacts;
+        const int p = local_ls ? i
+                               : i / kRoundContacts * rstride +
+                                     ((q / kGrpPerWarp) * nblk + block) * kGrpPerWarp + q % kGrpPerWarp;
+        if (p >= nc) continue;
         const int slot = k * kThreads + tid;
         ContactLine L;
         if (pass > 0 && k < kLsCacheDepth) {
@@ -1877,11 +1973,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
   for (int i = tid; i < kMaxBodies * kAdjBodySlots; i += kThreads) (&s_bb[0][0])[i] = 0.0;
   __syncthreads();
   Barrier B{a.bar, (unsigned)nblk, a.status, a.poison, 0, 0u, (unsigned)blockIdx.x};
-  const int gtid = blockIdx.x * kThreads + tid;
-  const int gstride = nblk * kThreads;
+  // (warps numbered across the blocks, as in the forward solve)
   const int lane = tid & 31;
-  const int gwarp = gtid >> 5;
-  const int nwarps = gstride >> 5;
+  const int gwarp = (tid >> 5) * nblk + (int)blockIdx.x;
+  const int nwarps = nblk * kWarps;
+  const int gtid = gwarp * 32 + lane;
+  const int gstride = nblk * kThreads;
   const GridDev& g = a.g;
   const size_t cap = (size_t)a.G.cnodes_cap;
   float4* vRhs = a.vec + kVRhs * cap;
