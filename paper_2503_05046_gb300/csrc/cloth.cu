@@ -29,11 +29,12 @@ namespace mpmcr {
 
 namespace {
 
-__global__ void k_cloth_forces(Particles P, const int* __restrict__ slot_of,
+__global__ void k_cloth_forces(Particles P, const int* slot_of,
                                const int4* __restrict__ tris, const double* __restrict__ rest,
                                int n_tris, const DevGroup* __restrict__ groups,
                                const uint8_t* __restrict__ pinned, float* __restrict__ f,
                                long long stride) {
+  chain_begin();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_tris) return;
   const int4 tv = tris[t];
@@ -104,9 +105,9 @@ __global__ void k_pin_init(Particles P, const int* __restrict__ slot_of, const i
   for (int c = 0; c < 9; ++c) P.C(c)[sl] = 0.f;
 }
 
-__global__ void k_pins(Particles P, const int* __restrict__ slot_of, const int* __restrict__ ids,
-                       const float* __restrict__ v_pin, float* __restrict__ x_pin, int n_pins,
-                       int cap, float h) {
+__global__ void k_pins(Particles P, const int* slot_of, const int* __restrict__ ids,
+                       const float* __restrict__ v_pin, float* x_pin, int n_pins, int cap, float h) {
+  chain_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_pins) return;
   const int sl = slot_of[ids[j]];
@@ -155,8 +156,8 @@ void launch_cloth_forces(const Particles& P, const int* slot_of, const int4* tri
   // one warp per block: a mesh of a few thousand triangles then spreads over
   // as many SMs as it has warps, since each SM's FP64 pipe is narrow
   if (n_tris > 0)
-    k_cloth_forces<<<(n_tris + 31) / 32, 32, 0, s>>>(P, slot_of, tris, rest, n_tris, groups,
-                                                      pinned, f, stride);
+    launch_chained(k_cloth_forces, dim3((n_tris + 31) / 32), 32, 0, s, P, slot_of, tris, rest, n_tris, groups,
+                   pinned, f, stride);
 }
 
 void launch_pin_init(const Particles& P, const int* slot_of, const int* ids, const float* v_pin,
@@ -168,7 +169,7 @@ void launch_pin_init(const Particles& P, const int* slot_of, const int* ids, con
 void launch_pins(const Particles& P, const int* slot_of, const int* ids, const float* v_pin,
                  float* x_pin, int n_pins, int cap, float h, cudaStream_t s) {
   if (n_pins > 0)
-    k_pins<<<(n_pins + 127) / 128, 128, 0, s>>>(P, slot_of, ids, v_pin, x_pin, n_pins, cap, h);
+    launch_chained(k_pins, dim3((n_pins + 127) / 128), 128, 0, s, P, slot_of, ids, v_pin, x_pin, n_pins, cap, h);
 }
 
 }  // namespace mpmcr
