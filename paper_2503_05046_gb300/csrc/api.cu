@@ -1429,7 +1429,7 @@ mpm_status mpm_contact_adjoint(mpm_ctx* ctx, int32_t mem_kind, int64_t n, const 
   CU(cudaMemsetAsync(ctx->G.n_cnodes, 0, sizeof(int), s));
   CU(cudaMemsetAsync(ctx->adj_body, 0, kAdjBodySlots * kMaxBodies * sizeof(double), s));
   CU(cudaMemsetAsync(ctx->adj_out, 0, 4 * sizeof(float), s));
-  CU(launch_adjoint(a, ctx->adj_blocks, s));
+  CU(launch_adjoint(a, ctx->adj_blocks, ctx->cluster_blocks, cluster_contacts(ctx), s));
   CU(cudaMemsetAsync(ctx->bar, 0, kBarWords * sizeof(unsigned), s));
   CU(cudaMemsetAsync(ctx->G.n_cnodes, 0, sizeof(int), s));
   st = drain_status(ctx);
@@ -1687,9 +1687,8 @@ mpm_status mpm_backward(mpm_ctx* ctx, int32_t mem_kind, const float* x_bar, cons
       a.out = ctx->adj_out; a.gbar = ctx->bw_gbar; a.pbar = bar[1 - in]; a.slot_of = ctx->bw_slot;
       a.P = P; a.n_particles = (int)n;
       a.body_gbar = step_dyn ? ctx->bw_gbody : nullptr;
-      CU(cudaMemsetAsync(ctx->bar, 0, kBarWords * sizeof(unsigned), s));
-      CU(cudaMemsetAsync(ctx->G.n_cnodes, 0, sizeof(int), s));
-      CU(launch_adjoint(a, ctx->adj_blocks, s));
+      launch_clear_solve(ctx->bar, ctx->G.n_cnodes, s);
+      CU(launch_adjoint(a, ctx->adj_blocks, ctx->cluster_blocks, cluster_contacts(ctx), s));
       launch_grid_adjoint(ba, ctx->num_sms, s);
       launch_p2g_adjoint(ba, s);
       launch_reset_counters(ctx->G, ctx->C, ctx->bar, ctx->stats, s);

@@ -626,6 +626,14 @@ __global__ void k_reset_counters(GridArrays G, Contacts C, unsigned* bar, DevSta
   bar[1] = 0u;
 }
 
+// The barrier counters and the node list's length, which are zero between
+// solves, after a substep's solve and before its adjoint.
+__global__ void k_clear_solve(unsigned* bar, int* n_cnodes) {
+  chain_begin();
+  bar[threadIdx.x] = 0u;
+  if (threadIdx.x == 0) *n_cnodes = 0;
+}
+
 // ---- solutions of the taped substeps ---------------------------------------
 // After each recorded solve, the velocities of its contact nodes (the only
 // nodes the solve changes) are appended to a pool as (v.x, v.y, v.z, node),
@@ -732,6 +740,10 @@ void launch_p2g_adjoint(const BackwardArgs& a, cudaStream_t s) {
 void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, DevStats* stats,
                            cudaStream_t s) {
   k_reset_counters<<<1, 1, 0, s>>>(G, C, bar, stats);
+}
+
+void launch_clear_solve(unsigned* bar, int* n_cnodes, cudaStream_t s) {
+  launch_chained(k_clear_solve, dim3(1), kBarWords, 0, s, bar, n_cnodes);
 }
 
 void launch_tape_save(const GridDev& g, const GridArrays& G, int* counters, int2* recs, int rec_cap, float4* pool,

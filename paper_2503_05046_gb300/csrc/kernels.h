@@ -193,6 +193,7 @@ struct AdjointArgs {
   // per body (6): the cotangent of the impulse and of its moment that the
   // substep's contacts give the body (dynamic bodies, Eq. (3)); null: none
   const double* body_gbar;
+  int cluster_max;    // (set by the launch) contacts up to which the cluster works, -1: none
 };
 constexpr int kAdjointVectors = 13;
 // per-body adjoint accumulators: dL/dv_r through the bias (3), its moment
@@ -202,7 +203,8 @@ constexpr int kAdjointVectors = 13;
 // rotation of the body's orientation (3) and dL/domega through the lagged
 // normal impulse (3)
 constexpr int kAdjBodySlots = 19;
-cudaError_t launch_adjoint(const AdjointArgs& a, int grid_blocks, cudaStream_t s);
+cudaError_t launch_adjoint(const AdjointArgs& a, int grid_blocks, int cluster_blocks, int cluster_max,
+                           cudaStream_t s);
 const void* adjoint_kernel_ptr();
 
 // ---- backward.cu: adjoints of G2P, the grid update and P2G (mpm_backward)
@@ -222,6 +224,7 @@ struct BackwardArgs {
 void launch_g2p_adjoint(const BackwardArgs& a, cudaStream_t s);
 void launch_grid_adjoint(const BackwardArgs& a, int num_sms, cudaStream_t s);
 void launch_p2g_adjoint(const BackwardArgs& a, cudaStream_t s);
+void launch_clear_solve(unsigned* bar, int* n_cnodes, cudaStream_t s);
 void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, DevStats* stats,
                            cudaStream_t s);
 void launch_slot_map(const Particles& P, int n, int* slot_of, cudaStream_t s);

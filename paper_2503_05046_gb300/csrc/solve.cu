@@ -60,6 +60,11 @@ constexpr int kWarps = kThreads / 32;
 // 902 with 64, 823 with 32, 777 with 16; below, a warp's lanes would be idle).
 constexpr int kContactsPerBlock = 16;
 constexpr int kAdjContactsPerBlock = 16;  // adjoint: one contact per warp
+// Up to this many contacts the adjoint's blocks are one cluster (two contacts per
+// warp): three barriers per iteration, which cost most of it. 65,536 particles
+// pushed over 25 substeps, forward and backward: 22.3 -> 18.4 ms, 30,000: 14.1 ->
+// 13.2. Up to 16 contacts one block works alone.
+constexpr int kAdjClusterContacts = 512;
 // Up to this many contacts (one per thread) each block line-searches alone.
 constexpr int kLocalLsMax = kThreads;
 constexpr int kLsPoints = 8;
@@ -1953,17 +1958,26 @@ __device__ __forceinline__ void lambda_at(const float4* xh, const float4* xl, in
   }
 }
 
+//
+// kCluster: up to a.cluster_max contacts by the blocks of one thread-block cluster
+// (every conjugate-gradient iteration has three barriers, two of them
+// reductions), otherwise the cooperative launch.
+template <bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
   __shared__ DevBody s_body[kMaxBodies];
   __shared__ float s_red[kWarps][kRedWidth];
   __shared__ float2 s_tot[kRedWidth];
+  __shared__ float2 s_cpart[4][kRedWidth];  // cluster: block sums, a ring of four reductions
   __shared__ double s_bb[kMaxBodies][kAdjBodySlots];  // FP64: the per-body sums cancel strongly
+  chain_begin();
   const int tid = threadIdx.x;
   // the last substep's contact count (G2P has reset the live counter), or
   // in mpm_backward mode the live count of the substep just solved
   const int count = a.gbar ? *a.C.count : a.stats->last_contacts;
   const int nc = count < a.C.cap ? count : a.C.cap;
+  if (kCluster ? nc > a.cluster_max : nc <= a.cluster_max) return;  // the other launch's
   int nblk = (nc + kAdjContactsPerBlock - 1) / kAdjContactsPerBlock;
+  nblk = kCluster && nblk > 1 ? (int)gridDim.x : nblk;  // (one block needs no cluster barrier)
   nblk = nblk < (int)gridDim.x ? nblk : (int)gridDim.x;
   nblk = nblk < kMaxSolveBlocks ? nblk : kMaxSolveBlocks;
   nblk = nblk > 1 ? nblk : 1;
@@ -1972,7 +1986,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
     reinterpret_cast<float*>(s_body)[i] = reinterpret_cast<const float*>(a.bodies)[i];
   for (int i = tid; i < kMaxBodies * kAdjBodySlots; i += kThreads) (&s_bb[0][0])[i] = 0.0;
   __syncthreads();
-  Barrier B{a.bar, (unsigned)nblk, a.status, a.poison, 0, 0u, (unsigned)blockIdx.x};
+  Barrier B{a.bar, (unsigned)nblk, a.status, a.poison, kCluster && nblk > 1 ? 1 : 0, 0u,
+            (unsigned)blockIdx.x};
   // (warps numbered across the blocks, as in the forward solve)
   const int lane = tid & 31;
   const int gwarp = (tid >> 5) * nblk + (int)blockIdx.x;
@@ -1999,6 +2014,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
     ++rslot;
     return s;
   };
+  int cslot = 0;
+  auto next_cpart = [&]() -> float2* { return kCluster ? s_cpart[(cslot++) & 3] : nullptr; };
   const int n_nodes_total = g.rx * g.ry * g.rz;
   auto node_of_id = [&](int id) -> int {
     if (id < 0 || id >= n_nodes_total) return -1;
@@ -2025,42 +2042,32 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
 
   // ---- contact-node list; flags hold list position + 1 (-1: claimed, no room)
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int p = gtid; p < nc; p += gstride) {
-    const float4 xp = a.C.xp[p];
-    Stencil s;
-    stencil(g, xp.x, xp.y, xp.z, s);
-    int node[27];
-    unsigned won = 0u;
-#pragma unroll
-    for (int c = 0; c < 27; ++c) {
-      node[c] = node_index(g, s.base[0] + c % 3, s.base[1] + (c / 3) % 3, s.base[2] + c / 9);
-      if (atomicCAS(a.G.cflag + node[c], 0, -1) == 0) won |= 1u << c;
-    }
+  for (int p = gwarp; p < nc; p += nwarps) {
+    const LaneNode ln = lane_node(g, a.C.xp[p], lane);
+    const bool won = lane < 27 && atomicCAS(a.G.cflag + ln.node, 0, -1) == 0;
+    const unsigned mask = __ballot_sync(0xffffffffu, won);
+    int slot0 = 0;
+    if (lane == 0 && mask) slot0 = atomicAdd(a.G.n_cnodes, __popc(mask));
+    const int slot = __shfl_sync(0xffffffffu, slot0, 0) + __popc(mask & ((1u << lane) - 1u));
     if (won) {
-      int slot = atomicAdd(a.G.n_cnodes, __popc(won));
-#pragma unroll
-      for (int c = 0; c < 27; ++c)
-        if ((won >> c) & 1u) {
-          if (slot < a.G.cnodes_cap) {
-            a.G.cnodes[slot] = node[c];
-            a.G.cflag[node[c]] = slot + 1;
-            if (a.gbar) {
-              const float4 gb = a.gbar[node[c]];
-              vRhs[slot] = make_float4(gb.x, gb.y, gb.z, 0.f);
-            } else {
-              vRhs[slot] = zero4;
-            }
-            vL0[slot] = zero4;
-            vL1[slot] = zero4;
-            vAcc[slot] = zero4;
-            double* d = acc64 + 4 * (size_t)slot;
-            d[0] = d[1] = d[2] = d[3] = 0.0;
-          } else {  // unreachable (the list holds every grid node): flag and clean up
-            atomicOr(a.status, kStCapacity);
-            atomicExch(a.poison, 1);
-          }
-          ++slot;
+      if (slot < a.G.cnodes_cap) {
+        a.G.cnodes[slot] = ln.node;
+        a.G.cflag[ln.node] = slot + 1;
+        if (a.gbar) {
+          const float4 gb = a.gbar[ln.node];
+          vRhs[slot] = make_float4(gb.x, gb.y, gb.z, 0.f);
+        } else {
+          vRhs[slot] = zero4;
         }
+        vL0[slot] = zero4;
+        vL1[slot] = zero4;
+        vAcc[slot] = zero4;
+        double* d = acc64 + 4 * (size_t)slot;
+        d[0] = d[1] = d[2] = d[3] = 0.0;
+      } else {  // unreachable (the list holds every grid node): flag and clean up
+        atomicOr(a.status, kStCapacity);
+        atomicExch(a.poison, 1);
+      }
     }
   }
   if (!grid_sync(B)) return;
@@ -2145,7 +2152,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
       vXh[t] = zero4;
       vXl[t] = zero4;
     }
-    if (!reduce_all(acc, next_slot(), B, s_red, s_tot)) return;
+    if (!reduce_all(acc, next_slot(), B, s_red, s_tot, next_cpart())) return;
   }
   const float rz_ref = s_tot[0].x + s_tot[0].y;  // |vbar|^2 in the P^-1 norm
   const float tol2 = (float)(a.eps_r * a.eps_r) * rz_ref;
@@ -2232,7 +2239,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
           vP[t] = pp;
           vQ[t] = q;
         }
-        if (!reduce_all(acc, next_slot(), B, s_red, s_tot)) return;
+        if (!reduce_all(acc, next_slot(), B, s_red, s_tot, next_cpart())) return;
       }
       const float pq = s_tot[0].x + s_tot[0].y;
       if (!(pq > 0.f)) {  // H^ is positive definite on the free DoFs: only rounding gets here
@@ -2256,7 +2263,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
           vZ[t] = z;
           acc[0] += r.x * z.x + r.y * z.y + r.z * z.z;
         }
-        if (!reduce_all(acc, next_slot(), B, s_red, s_tot)) return;
+        if (!reduce_all(acc, next_slot(), B, s_red, s_tot, next_cpart())) return;
       }
       const float rz_new = s_tot[0].x + s_tot[0].y;
       beta = rz > 0.f ? rz_new / rz : 0.f;
@@ -2312,7 +2319,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
         vZ[t] = z;
         acc[0] += r.x * z.x + r.y * z.y + r.z * z.z;
       }
-      if (!reduce_all(acc, next_slot(), B, s_red, s_tot)) return;
+      if (!reduce_all(acc, next_slot(), B, s_red, s_tot, next_cpart())) return;
     }
     rz_true = s_tot[0].x + s_tot[0].y;
     rz = rz_true;
@@ -2492,6 +2499,9 @@ cudaError_t solve_prepare() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_solve<true>),
                              cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_adjoint<true>),
+                             cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   for (const void* f : {reinterpret_cast<const void*>(&k_solve_small),
                         reinterpret_cast<const void*>(&k_solve_small_batch)})
     if (e == cudaSuccess)
@@ -2584,12 +2594,22 @@ cudaError_t launch_solve_batch(const SolveArgs* args, const int* order, int n_sc
   }
 }
 
-const void* adjoint_kernel_ptr() { return reinterpret_cast<const void*>(&k_adjoint); }
+const void* adjoint_kernel_ptr() { return reinterpret_cast<const void*>(&k_adjoint<false>); }
 
-cudaError_t launch_adjoint(const AdjointArgs& a, int grid_blocks, cudaStream_t s) {
+cudaError_t launch_adjoint(const AdjointArgs& a, int grid_blocks, int cluster_blocks, int cluster_max,
+                           cudaStream_t s) {
   AdjointArgs args = a;
+  args.cluster_max = -1;
+  if (cluster_blocks > 0 && cluster_max > 0) {
+    args.cluster_max = cluster_max < kAdjClusterContacts ? cluster_max : kAdjClusterContacts;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(cluster_blocks, attr, s);
+    cfg.dynamicSmemBytes = 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_adjoint<true>, args);
+    if (e != cudaSuccess) return e;
+  }
   void* params[] = {&args};
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_adjoint), dim3(grid_blocks),
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_adjoint<false>), dim3(grid_blocks),
                                      dim3(kThreads), params, 0, s);
 }
 
