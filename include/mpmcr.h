@@ -517,7 +517,8 @@ mpm_status mpm_synchronize(mpm_ctx* ctx);
    solved by one thread-block cluster (up to 16 SMs exchanging their sums
    through distributed shared memory, hardware cluster barriers); more
    contacts go to the cooperative launch over as many SMs as they need, with
-   device-wide barriers (default 1024; 0: always the cooperative launch).
+   device-wide barriers (unset: 4096, and 1024 from 160,000 particles on; 0:
+   always the cooperative launch).
    MPM_OPT_CLUSTER_BLOCKS: thread blocks (SMs) in that cluster, a power of two
    up to the largest the device schedules (0, the default: the largest, 16 on
    GB300).
@@ -556,14 +557,14 @@ mpm_status mpm_get_phase_times(mpm_ctx* ctx, double* ms, int64_t* launches, int3
    Launch overhead dominates small scenes (Sec. V-A: the per-substep kernel
    launches and host-device synchronisations). A batch advances n
    independent contexts together so that one substep of ALL of them costs
-   five launches: P2G (with contact registration), grid
-   update, contact solve (Alg. 1) and G2P, each over a work list of
-   (scene, thread block) items that covers every scene, plus one launch at
-   the start and one at the end of the time step (the latter moves every
-   scene's bodies on the device as mpm_step does, Eq. (3)-(4)). The time
-   step replays as one CUDA graph. Each scene's contact solve runs in one
-   thread block (or one thread-block cluster) of its own: its reductions need
-   no device-wide barrier.
+   five launches: P2G (with contact registration), grid update, contact solve
+   (Alg. 1; one launch for scenes of few contacts and one for the others) and
+   G2P, each over a work list of (scene, thread block) items that covers every
+   scene, plus one launch at the start and one at the end of the time step
+   (the latter moves every scene's bodies on the device as mpm_step does,
+   Eq. (3)-(4)). The time step replays as one CUDA graph. Each scene's contact
+   solve runs in one thread block (or one thread-block cluster) of its own:
+   its reductions need no device-wide barrier.
 
    Members are contexts created on the same device with the SAME
    cuda_stream (the batch's stream), none recording a tape; the caller keeps

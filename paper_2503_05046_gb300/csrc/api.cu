@@ -371,9 +371,19 @@ void release(mpm_ctx* c) {
 }
 
 // Contact counts up to which one thread-block cluster solves (the barrier
-// time-limit test needs the cooperative kernel's device-wide barriers).
+// time-limit test needs the cooperative kernel's device-wide barriers). Alone on
+// the device, cluster and cooperative launch cross at about 1,000 contacts
+// (contact solve of a step of ten substeps, us: 402 contacts 254 and 277, 1,026 on
+// a slab 255 and 282, 926 spread out 427 and 395, 1,543 spread out 609 and 474,
+// 3,105 1,284 and 706). But cooperative launches of several contexts do not run
+// side by side: 128 scenes of 2k to 64k particles, a context and a stream each,
+// make 5,561 scene-steps/s with clusters up to 4,096 contacts and 3,141 with 1,024.
+// So the crossing holds for contexts whose transfers fill the device, and 4,096 for
+// smaller ones, which may share it.
 int cluster_contacts(const mpm_ctx* ctx) {
-  return ctx->wait_test || ctx->cluster_blocks == 0 ? 0 : ctx->cluster_max;
+  if (ctx->wait_test || ctx->cluster_blocks == 0) return 0;
+  if (ctx->cluster_max >= 0) return ctx->cluster_max;
+  return ctx->n >= 160000 ? 1024 : 4096;
 }
 
 // One substep on particle buffer `cur`: P2G, grid update, contact solve and

@@ -20,11 +20,7 @@ struct mpm_ctx {
   int num_sms = 0, solve_blocks = 0;
   int cluster_blocks = 0;     // blocks of the cluster solve (0: the device runs none)
   int cluster_blocks_max = 0; // the largest cluster the device schedules
-  // MPM_OPT_CLUSTER_CONTACTS: where the cluster and the cooperative launch cross
-  // (contact solve of a step of ten substeps, us: 402 contacts 254 and 277, 1,026
-  // on a slab 255 and 282, 926 spread out 427 and 395, 1,543 spread out 609 and
-  // 474, 3,105 1,284 and 706)
-  int cluster_max = 1024;
+  int cluster_max = -1;       // MPM_OPT_CLUSTER_CONTACTS (negative: not set)
   float* pbuf[2] = {nullptr, nullptr};
   uint32_t* pidbuf[2] = {nullptr, nullptr};
   uint16_t* grpbuf[2] = {nullptr, nullptr};
