@@ -6,13 +6,13 @@ the timed steps are ordinary steps of the simulation):
 
 - a batch (native.Batch, mpm_batch_*): one launch per phase per substep over
   all scenes' (scene, block) work items. `tune_batch_launch` picks the
-  particles per P2G warp tile (MPM_BATCH_OPT_P2G_CHUNK / 8 warps), the
+  particles per P2G block (MPM_BATCH_OPT_P2G_CHUNK: without effect), the
   threads per G2P block, the particles per grid-phase block and the blocks
   per scene's contact solve, by coordinate descent;
 - contexts side by side, each on its own stream replaying its step's CUDA
   graph (mpm_step with graphs on). `tune_batch` picks the cap on the SMs one
   context's cooperative contact solve occupies (MPM_OPT_SOLVE_BLOCKS) and the
-  particles per P2G thread block (MPM_OPT_P2G_CHUNK).
+  particles per P2G thread block (MPM_OPT_P2G_CHUNK: without effect).
 """
 import time
 
@@ -98,13 +98,13 @@ def tune_batch_launch(batch, h, n_substeps, solver, steps=2, p2g_chunks=(256, 51
 
 def tune_p2g_form(sim, solver, steps=1, candidates=((0, 256), (0, 1024), (1, 256))):
     """Time the P2G launches of `steps` steps of one context for each
-    (form, particles per block) candidate: the gather form (0) at 256 and
-    1,024 particles per block, the scatter form (1) at 256 (phase events, so
+    (form, particles per block) candidate (phase events, so
     that the comparison does not depend on how the rest of the steps, which
     advance the simulation, differ). Apply and return the fastest
     (form, chunk) and the table of ((form, chunk), P2G milliseconds per
-    launch). The gather form wins at several particles per cell, the scatter
-    form near one."""
+    launch). The library accepts both options without effect: one P2G serves
+    every particle density, so the times differ by their noise and by how far
+    the steps have come."""
     table = []
     native.mpm_set_option(sim.ctx, native.OPT_PROFILE, 1)
     try:
