@@ -64,10 +64,13 @@ __global__ void k_cloth_forces(Particles P, const int* slot_of,
   if (!(detC > 1e-30)) return;  // a collapsed triangle exerts no force
   const double J = sqrt(detC);
   const double tn = sqrt(c00 + c11 + 2.0 * J);
-  const double s00 = (c00 + J) / tn, s01 = c01 / tn, s11 = (c11 + J) / tn;
+  // (an FP64 division is some twenty instructions of a pipe that takes sixteen
+  // cycles for each: one per denominator. 1,682 triangles: 11.2 -> 8.9 us)
+  const double itn = 1.0 / tn, iJ = 1.0 / J, idet = 1.0 / detC;
+  const double s00 = (c00 + J) * itn, s01 = c01 * itn, s11 = (c11 + J) * itn;
   // R = F S^-1 (det S = J); P = 2 mu (F - R) + lam (J - 1) J F C^-1
-  const double si00 = s11 / J, si01 = -s01 / J, si11 = s00 / J;
-  const double ci00 = c11 / detC, ci01 = -c01 / detC, ci11 = c00 / detC;
+  const double si00 = s11 * iJ, si01 = -s01 * iJ, si11 = s00 * iJ;
+  const double ci00 = c11 * idet, ci01 = -c01 * idet, ci11 = c00 * idet;
   const double kl = lam * (J - 1.0) * J;
   double g[3][2];
 #pragma unroll
