@@ -391,7 +391,7 @@ __device__ __forceinline__ void load_contact(const Contacts& C, int p, float4& x
 // line form in shared-memory slot k * kThreads + tid across the passes of one
 // line search, packed into three float4: (v_n, e_n, vhat, phi0),
 // (mu n0, body, v_t.x, v_t.y), (v_t.z, e_t); k and d come from the body table.
-constexpr int kLsCacheDepth = 2;  // (four took the L1 more than it saved)
+constexpr int kLsCacheDepth = 2;  // (one and four measured the same; four is 49 KB more)
 constexpr int kLsCacheSlots = kLsCacheDepth * kThreads;
 
 __device__ __forceinline__ void line_store(float4* cache, int slot, const ContactLine& L, int body) {
