@@ -198,8 +198,11 @@ __device__ __forceinline__ int active_with_storage(const GridDev& g, int n_act) 
 // First statement of every kernel launched by launch_chained: waits until the
 // kernel before it on the stream is complete and its writes are visible, then
 // lets the next one's blocks be set up beside this one's. (Their loads must not
-// pass the wait: what a kernel of the chain reads of an earlier one's is not
-// read through a const __restrict__ parameter, which the compiler may hoist.)
+// pass the wait, nor be served from before it: what a kernel of the chain reads
+// of an earlier one's goes through ordinary loads, never through __ldg or a
+// const __restrict__ parameter. Such a load is defined only for data that stays
+// unwritten for the whole life of the kernel, which begins before the wait, and
+// the compiler may hoist it.)
 __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

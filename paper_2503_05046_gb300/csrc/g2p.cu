@@ -80,7 +80,7 @@ __device__ __forceinline__ void g2p_block(const G2PArgs& a, int block) {
         const float w = s.w[0][cx] * wyz;
         const int node = kDense ? az[cz] + ay[cy] + ax[cx]
                                 : node_index(g, s.base[0] + cx, s.base[1] + cy, s.base[2] + cz);
-        const float4 v = __ldg(a.G.v + node);
+        const float4 v = a.G.v[node];  // (the solve before writes it: no read-only load)
         const float2 wv = __fmul2_rn(make_float2(w, w), make_float2(v.x, v.y));
         const float wvz = w * v.z;
         Sxy = __fadd2_rn(Sxy, wv);

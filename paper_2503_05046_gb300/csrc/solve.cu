@@ -2360,7 +2360,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_adjoint(AdjointArgs a) {
       lane_weight_grad(g, xp, lane, gw);
       double lam[3];
       lambda_at(vXh, vXl, ci, lam);
-      const float4 vi = lane < 27 ? __ldg(a.G.v + ln.node) : zero4;
+      const float4 vi = lane < 27 ? a.G.v[ln.node] : zero4;
       double gc[3];
 #pragma unroll
       for (int r = 0; r < 3; ++r) gc[r] = (double)A.dN * A.n[r] + (double)A.cs * A.ut[r];
