@@ -517,7 +517,9 @@ mpm_status mpm_synchronize(mpm_ctx* ctx);
    solved by one thread-block cluster (up to 16 SMs exchanging their sums
    through distributed shared memory, hardware cluster barriers); more
    contacts go to the cooperative launch over as many SMs as they need, with
-   device-wide barriers (unset: 4096, and 1024 from 160,000 particles on; 0:
+   device-wide barriers (unset: 4096; a context of at least 160,000 particles
+   takes 1024 instead in each substep that finds no other context's step in
+   flight on the device, since cooperative launches do not run side by side; 0:
    always the cooperative launch).
    MPM_OPT_CLUSTER_BLOCKS: thread blocks (SMs) in that cluster, a power of two
    up to the largest the device schedules (0, the default: the largest, 16 on

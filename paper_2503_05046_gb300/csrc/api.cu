@@ -370,34 +370,54 @@ void release(mpm_ctx* c) {
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
 }
 
+// Steps in flight on this device, counted by the device itself: the first P2G of
+// a step adds one, its last G2P takes it off again (a batch's step and each
+// substep that a backward pass replays count as one too).
+__device__ int g_steps_in_flight;
+
 // Contact counts up to which one thread-block cluster solves (the barrier
 // time-limit test needs the cooperative kernel's device-wide barriers). Alone on
 // the device, cluster and cooperative launch cross at about 1,000 contacts
 // (contact solve of a step of ten substeps, us: 402 contacts 254 and 277, 1,026 on
 // a slab 255 and 282, 926 spread out 427 and 395, 1,543 spread out 609 and 474,
-// 3,105 1,284 and 706). But cooperative launches of several contexts do not run
-// side by side: 128 scenes of 2k to 64k particles, a context and a stream each,
-// make 5,561 scene-steps/s with clusters up to 4,096 contacts and 3,141 with 1,024.
-// So the crossing holds for contexts whose transfers fill the device, and 4,096 for
-// smaller ones, which may share it.
+// 3,105 1,284 and 706). Cooperative launches of several contexts do not run side
+// by side, small or large: each waits until every SM is free. A step's us per
+// scene with 1, 2, 4 and 8 contexts, a stream each, cluster up to 4,096 contacts
+// and up to 1,024:
+//   160,000 sand in a slab, 1,600 contacts      759   448   332   301 |   787   602   517   519
+//   360,000 sand in a slab, 3,600 contacts    1,039   737   591   556 |   947   882   883   859
+//   600,000 sand scooped,   1,851 contacts    2,330 1,849 1,531 1,461 | 2,164 1,902 1,913 1,842
+//   1M sand scooped,        3,073 contacts    3,555 2,784 2,286 2,106 | 3,004 2,739 2,820 2,628
+// (Capping that launch's blocks does not mend it: 38 blocks 580 and 443 us with two
+// and four slabs of 160,000.) So the crossing holds for a context that fills the
+// device by its transfers and has it to itself, 4,096 for all others: from 160,000
+// particles on, cluster_contacts_alone() holds for the substeps whose solve finds
+// no other step in flight (with it, in the same four counts: 789 456 340 309, 946
+// 784 599 567, 2,096 1,876 1,547 1,430 and 2,968 2,795 2,290 2,110).
 int cluster_contacts(const mpm_ctx* ctx) {
   if (ctx->wait_test || ctx->cluster_blocks == 0) return 0;
-  if (ctx->cluster_max >= 0) return ctx->cluster_max;
-  return ctx->n >= 160000 ? 1024 : 4096;
+  return ctx->cluster_max >= 0 ? ctx->cluster_max : 4096;
+}
+
+int cluster_contacts_alone(const mpm_ctx* ctx) {
+  const int all = cluster_contacts(ctx);
+  return all > 0 && ctx->cluster_max < 0 && ctx->n >= 160000 ? 1024 : all;
 }
 
 // One substep on particle buffer `cur`: P2G, grid update, contact solve and
 // (with_g2p) G2P. save: append the solve's contact-node velocities to the
 // tape's solution pool; warm_rec >= 0: start the solve from the taped
-// solution record warm_rec instead of v*.
+// solution record warm_rec instead of v*. first, last: of its step (both for a
+// substep by itself; without G2P the caller ends it by launch_reset_counters).
 cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_solver_params& sp,
                             int solve_blocks, bool with_g2p, cudaStream_t s, bool save = false,
-                            int warm_rec = -1) {
+                            int warm_rec = -1, bool first = true, bool last = true) {
   const int n = (int)ctx->n;
   P2GArgs pa;
   pa.g = ctx->g; pa.P = ctx->P[cur]; pa.n = n; pa.groups = ctx->groups_d;
   pa.bodies = ctx->bodies_d; pa.nb = nb; pa.h = hf; pa.G = ctx->G; pa.C = ctx->C;
   pa.status = ctx->status; pa.stats = ctx->stats;
+  pa.in_flight = first ? ctx->in_flight : nullptr;
   pa.fext = nullptr;
   pa.fext_stride = ctx->cap;
   if (!ctx->cloth_tris.empty()) {
@@ -427,6 +447,8 @@ cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_s
   sa.wait_extra = ctx->wait_test ? 1 : 0;
   sa.poison = ctx->poison;
   sa.cluster_max = cluster_contacts(ctx);
+  sa.cluster_alone = cluster_contacts_alone(ctx);
+  sa.in_flight = ctx->in_flight;
   sa.small_max = 0;  // (set by the launch)
   mark_phase(ctx, MPM_PHASE_SOLVE);
   const cudaError_t e = launch_solve(sa, solve_blocks, ctx->cluster_blocks, s);
@@ -438,6 +460,7 @@ cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_s
     G2PArgs ga;
     ga.g = ctx->g; ga.P = ctx->P[cur]; ga.n = n; ga.groups = ctx->groups_d; ga.G = ctx->G;
     ga.C = ctx->C; ga.h = hf; ga.bar = ctx->bar; ga.red = ctx->red; ga.stats = ctx->stats;
+    ga.in_flight = last && n > 0 ? ctx->in_flight : nullptr;  // (no particles: P2G launches nothing)
     mark_phase(ctx, MPM_PHASE_G2P);
     launch_g2p(ga, s);
     launch_pins(ctx->P[cur], ctx->slot_of_d, ctx->pin_ids_d, ctx->pin_v_d, ctx->pin_x_d, ctx->n_pins,
@@ -476,7 +499,8 @@ cudaError_t enqueue_step(mpm_ctx* ctx, int from, bool sort_now, int n_substeps, 
     launch_pin_init(ctx->P[cur], ctx->slot_of_d, ctx->pin_ids_d, ctx->pin_v_d, ctx->pin_x_d,
                     ctx->n_pins, ctx->pins_cap, s);
   for (int k = 0; k < n_substeps; ++k) {
-    const cudaError_t e = enqueue_substep(ctx, cur, nb, hf, sp, solve_blocks, true, s, ctx->taping);
+    const cudaError_t e = enqueue_substep(ctx, cur, nb, hf, sp, solve_blocks, true, s, ctx->taping, -1,
+                                          k == 0, k == n_substeps - 1);
     if (e != cudaSuccess) return e;
   }
   if (rigid && nb > 0) {
@@ -697,6 +721,9 @@ mpm_status mpm_create(const mpm_grid_spec* spec, void* cuda_stream, mpm_ctx** ou
   ctx->solve_blocks = ctx->num_sms * (occ < 2 ? occ : 2);
   ctx->cluster_blocks = solve_cluster_blocks();
   ctx->cluster_blocks_max = ctx->cluster_blocks;
+  void* counter = nullptr;
+  if (cudaGetSymbolAddress(&counter, g_steps_in_flight) != cudaSuccess) return bail(MPM_ERR_CUDA);
+  ctx->in_flight = static_cast<int*>(counter);
   *out = ctx;
   return MPM_OK;
 }
@@ -1149,6 +1176,7 @@ mpm_status mpm_step(mpm_ctx* ctx, double h, int32_t n_substeps, const mpm_solver
     k.n = n; k.n_substeps = n_substeps; k.nb = nb; k.chunk = ctx->p2g_chunk;
     k.sort_now = sort_now ? 1 : 0; k.solve_blocks = solve_blocks; k.h = hf; k.sp = sp;
     k.cluster_max = cluster_contacts(ctx);
+    k.cluster_alone = cluster_contacts_alone(ctx);
     k.cluster_blocks = ctx->cluster_blocks;
     k.p2g_form = ctx->p2g_form;
     k.rigid = dev_rigid ? 1 : 0;
@@ -1158,7 +1186,8 @@ mpm_status mpm_step(mpm_ctx* ctx, double h, int32_t n_substeps, const mpm_solver
     const bool same = ctx->gexec[from] && o.n == k.n && o.n_substeps == k.n_substeps && o.nb == k.nb &&
                       o.chunk == k.chunk && o.sort_now == k.sort_now &&
                       o.solve_blocks == k.solve_blocks && o.h == k.h && o.taping == k.taping &&
-                      o.cluster_max == k.cluster_max && o.cluster_blocks == k.cluster_blocks &&
+                      o.cluster_max == k.cluster_max && o.cluster_alone == k.cluster_alone &&
+                      o.cluster_blocks == k.cluster_blocks &&
                       o.rigid == k.rigid && o.p2g_form == k.p2g_form &&
                       o.tape_pool == k.tape_pool &&
                       memcmp(&o.sp, &k.sp, sizeof(k.sp)) == 0;
@@ -1701,7 +1730,7 @@ mpm_status mpm_backward(mpm_ctx* ctx, int32_t mem_kind, const float* x_bar, cons
       CU(launch_adjoint(a, ctx->adj_blocks, ctx->cluster_blocks, cluster_contacts(ctx), s));
       launch_grid_adjoint(ba, ctx->num_sms, s);
       launch_p2g_adjoint(ba, s);
-      launch_reset_counters(ctx->G, ctx->C, ctx->bar, ctx->stats, s);
+      launch_reset_counters(ctx->G, ctx->C, ctx->bar, ctx->stats, n > 0 ? ctx->in_flight : nullptr, s);
       CU(cudaGetLastError());
       in = 1 - in;
       ++substeps;

@@ -616,7 +616,9 @@ __global__ void __launch_bounds__(kThreads) k_p2g_adjoint(BackwardArgs a) {
 
 // The per-substep counters that G2P resets in the forward pass (the
 // backward replays P2G, grid and solve without G2P).
-__global__ void k_reset_counters(GridArrays G, Contacts C, unsigned* bar, DevStats* stats) {
+__global__ void k_reset_counters(GridArrays G, Contacts C, unsigned* bar, DevStats* stats,
+                                 int* in_flight) {
+  if (in_flight) atomicSub(in_flight, 1);
   stats->last_active = *G.n_act;
   *C.count = 0;
   *G.n_act = 0;
@@ -738,8 +740,8 @@ void launch_p2g_adjoint(const BackwardArgs& a, cudaStream_t s) {
 }
 
 void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, DevStats* stats,
-                           cudaStream_t s) {
-  k_reset_counters<<<1, 1, 0, s>>>(G, C, bar, stats);
+                           int* in_flight, cudaStream_t s) {
+  k_reset_counters<<<1, 1, 0, s>>>(G, C, bar, stats, in_flight);
 }
 
 void launch_clear_solve(unsigned* bar, int* n_cnodes, cudaStream_t s) {

@@ -212,7 +212,7 @@ int solve_blocks_of(const mpm_batch* b) {
 cudaError_t enqueue(mpm_batch* b, int n_substeps, double dt) {
   const cudaStream_t s = b->stream;
   const int ns = (int)b->ctx.size();
-  launch_batch_begin(b->rig_d, ns, s);
+  launch_batch_begin(b->rig_d, ns, b->ctx[0]->in_flight, s);
   for (int k = 0; k < n_substeps; ++k) {
     launch_p2g_batch(b->p2g_d, b->work_d, b->n_p2g, b->n_all, s);
     launch_grid_batch(b->grid_d, b->work_d + b->n_p2g, b->n_grid, s);
@@ -220,7 +220,7 @@ cudaError_t enqueue(mpm_batch* b, int n_substeps, double dt) {
     if (e != cudaSuccess) return e;
     launch_g2p_batch(b->g2p_d, b->work_d + b->n_p2g + b->n_grid, b->n_g2p, b->g2p_threads, s);
   }
-  launch_batch_end(b->rig_d, ns, dt, b->status_d, b->stats_d, s);
+  launch_batch_end(b->rig_d, ns, dt, b->status_d, b->stats_d, b->ctx[0]->in_flight, s);
   return cudaGetLastError();
 }
 

@@ -21,6 +21,7 @@ struct mpm_ctx {
   int cluster_blocks = 0;     // blocks of the cluster solve (0: the device runs none)
   int cluster_blocks_max = 0; // the largest cluster the device schedules
   int cluster_max = -1;       // MPM_OPT_CLUSTER_CONTACTS (negative: not set)
+  int* in_flight = nullptr;   // the device's count of steps in flight
   float* pbuf[2] = {nullptr, nullptr};
   uint32_t* pidbuf[2] = {nullptr, nullptr};
   uint16_t* grpbuf[2] = {nullptr, nullptr};
@@ -83,7 +84,7 @@ struct mpm_ctx {
   struct GraphKey {
     int64_t n = -1;
     int n_substeps = 0, nb = 0, chunk = 0, sort_now = 0, solve_blocks = 0, taping = 0;
-    int cluster_max = 0;
+    int cluster_max = 0, cluster_alone = 0;
     int cluster_blocks = 0;
     int p2g_form = 0;
     int rigid = 0;

@@ -41,6 +41,7 @@ __device__ __forceinline__ void g2p_block(const G2PArgs& a, int block) {
       *a.G.n_act = 0;
       *a.G.n_cnodes = 0;
       *a.G.pstar2 = 0.0;
+      if (a.in_flight) atomicSub(a.in_flight, 1);
     }
     if (threadIdx.x < 2) a.bar[threadIdx.x] = 0u;  // the solve's 64-bit barrier counter
   }

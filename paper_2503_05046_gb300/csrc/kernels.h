@@ -110,6 +110,7 @@ struct P2GArgs {
   Contacts C;
   uint32_t* status;
   DevStats* stats;
+  int* in_flight;  // the step's first substep: the device's count of steps in flight, else null
   float* fext;  // cloth: per-particle mesh forces, 3 planes of fext_stride (null: none); P2G zeroes them
   long long fext_stride;
 };
@@ -144,6 +145,8 @@ struct SolveArgs {
   int wait_extra;     // 0; 1 makes every grid barrier wait for one block too many (test)
   int* poison;        // nonzero after a barrier gave up (set and cleared by the solve)
   int cluster_max;    // up to this many contacts one thread-block cluster solves (0: never)
+  int cluster_alone;  // the same while no other step is in flight on the device (<= cluster_max)
+  const int* in_flight;  // the device's count of steps in flight, this one among them
   int small_max;      // up to this many the one-block kernel may have solved (set by the launchers)
 };
 // the one-block and the cluster kernel (cluster_blocks > 0 and a.cluster_max > 0),
@@ -226,7 +229,7 @@ void launch_grid_adjoint(const BackwardArgs& a, int num_sms, cudaStream_t s);
 void launch_p2g_adjoint(const BackwardArgs& a, cudaStream_t s);
 void launch_clear_solve(unsigned* bar, int* n_cnodes, cudaStream_t s);
 void launch_reset_counters(const GridArrays& G, const Contacts& C, unsigned* bar, DevStats* stats,
-                           cudaStream_t s);
+                           int* in_flight, cudaStream_t s);
 void launch_slot_map(const Particles& P, int n, int* slot_of, cudaStream_t s);
 // taped solutions: append the contact-node velocities after a solve (counters:
 // [0] pool fill, [1] records written); scatter record r over v*
@@ -290,9 +293,9 @@ struct RigidBatchArgs {
   const uint32_t* status;
   double gravity[3];
 };
-void launch_batch_begin(const RigidBatchArgs* args, int n_scenes, cudaStream_t s);
+void launch_batch_begin(const RigidBatchArgs* args, int n_scenes, int* in_flight, cudaStream_t s);
 void launch_batch_end(const RigidBatchArgs* args, int n_scenes, double dt, uint32_t* status_out,
-                      DevStats* stats_out, cudaStream_t s);
+                      DevStats* stats_out, int* in_flight, cudaStream_t s);
 
 // ---- g2p.cu: grid-to-particle with the constitutive update ----
 struct G2PArgs {
@@ -306,6 +309,7 @@ struct G2PArgs {
   unsigned* bar;     // solve barrier, reset here
   double* red;       // solve reduction ring, reset here
   DevStats* stats;
+  int* in_flight;    // the step's last substep: as P2GArgs', else null
 };
 void launch_g2p(const G2PArgs& a, cudaStream_t s);
 

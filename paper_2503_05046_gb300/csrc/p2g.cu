@@ -413,6 +413,7 @@ __device__ __forceinline__ void p2g_walk_block(const P2GArgs& a, int block) {
 template <int ROUNDS, bool kDense>
 __global__ void __launch_bounds__(kWalkThreads, 24) k_p2g_w(P2GArgs a) {
   chain_begin();
+  if (a.in_flight && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(a.in_flight, 1);
   p2g_walk_block<ROUNDS, kDense>(a, blockIdx.x);
 }
 

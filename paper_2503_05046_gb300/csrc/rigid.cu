@@ -143,7 +143,8 @@ __global__ void k_rigid_update(DevBody* bodies, const DevDyn* dyn, int nb, const
 
 // Batched, block s for scene s: the step's start (its statistics cleared,
 // the impulse accumulator noted) ...
-__global__ void k_batch_begin(const RigidBatchArgs* __restrict__ args) {
+__global__ void k_batch_begin(const RigidBatchArgs* __restrict__ args, int* in_flight) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(in_flight, 1);
   const RigidBatchArgs& a = args[blockIdx.x];
   for (int i = threadIdx.x; i < (int)(sizeof(DevStats) / 4); i += blockDim.x)
     reinterpret_cast<int*>(a.stats)[i] = 0;
@@ -153,7 +154,9 @@ __global__ void k_batch_begin(const RigidBatchArgs* __restrict__ args) {
 // ... and its end: one warp per body moves the bodies, and the scene's
 // status word and statistics are gathered into the batch's arrays
 __global__ void k_batch_end(const RigidBatchArgs* __restrict__ args, double dt,
-                            uint32_t* __restrict__ status_out, DevStats* __restrict__ stats_out) {
+                            uint32_t* __restrict__ status_out, DevStats* __restrict__ stats_out,
+                            int* in_flight) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicSub(in_flight, 1);
   const RigidBatchArgs& a = args[blockIdx.x];
   if (threadIdx.x == 0) status_out[blockIdx.x] = *a.status;
   for (int i = threadIdx.x; i < (int)(sizeof(DevStats) / 4); i += blockDim.x)
@@ -166,14 +169,14 @@ __global__ void k_batch_end(const RigidBatchArgs* __restrict__ args, double dt,
 
 }  // namespace
 
-void launch_batch_begin(const RigidBatchArgs* args, int n_scenes, cudaStream_t s) {
-  if (n_scenes > 0) k_batch_begin<<<n_scenes, 128, 0, s>>>(args);
+void launch_batch_begin(const RigidBatchArgs* args, int n_scenes, int* in_flight, cudaStream_t s) {
+  if (n_scenes > 0) k_batch_begin<<<n_scenes, 128, 0, s>>>(args, in_flight);
 }
 
 void launch_batch_end(const RigidBatchArgs* args, int n_scenes, double dt, uint32_t* status_out,
-                      DevStats* stats_out, cudaStream_t s) {
+                      DevStats* stats_out, int* in_flight, cudaStream_t s) {
   if (n_scenes > 0)
-    k_batch_end<<<n_scenes, 32 * kMaxBodies, 0, s>>>(args, dt, status_out, stats_out);
+    k_batch_end<<<n_scenes, 32 * kMaxBodies, 0, s>>>(args, dt, status_out, stats_out, in_flight);
 }
 
 void launch_rigid_update(DevBody* bodies, const DevDyn* dyn, int nb, const double* imp,

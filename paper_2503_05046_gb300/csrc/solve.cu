@@ -659,6 +659,7 @@ __device__ __forceinline__ void solve_stats(const SolveArgs& a, const unsigned l
 // It sets a flag that the other solve kernels of the substep test.
 constexpr int kSmallContacts = 320;
 constexpr int kSmallFlag = 16;      // word of SolveArgs::bar: 1 if the one-block kernel solved the substep
+constexpr int kRouteWord = 17;      // another: up to how many contacts the cluster solves this substep
 constexpr int kSmallHash = 8192;    // slots of the node hash table (128 blocks of 64)
 constexpr int kSmallNodes = 4096;   // most nodes (half of the table)
 constexpr int kSmallProbes = 32;
@@ -734,6 +735,10 @@ __device__ __forceinline__ void small_solve(const SolveArgs& a) {
   int* s_warp = reinterpret_cast<int*>(&s_red[0][0]);
   const int count = *a.C.count;
   const int nc = count < a.C.cap ? count : a.C.cap;
+  // (the cluster and the cooperative kernel have to agree on the route: it is
+  // chosen here for both)
+  if (a.cluster_alone < a.cluster_max && tid == 0)
+    a.bar[kRouteWord] = (unsigned)(__ldcg(a.in_flight) > 1 ? a.cluster_max : a.cluster_alone);
   if (nc == 0 || nc > a.small_max || __ldcg(a.poison)) {
     if (tid == 0) a.bar[kSmallFlag] = 0u;
     return;
@@ -1175,7 +1180,10 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   if (nc == 0) return;  // v = v* already (set by the grid update)
   // (every block of a launch reads the same count: the choice is uniform)
   if (nc <= a.small_max && __ldcg(a.bar + kSmallFlag)) return;  // solved by the one-block kernel
-  if (kCluster ? nc > a.cluster_max : nc <= a.cluster_max) return;  // the other kernel's
+  const int cluster_max = nc > a.cluster_alone && nc <= a.cluster_max
+                              ? (int)__ldcg(a.bar + kRouteWord)  // (the one-block kernel has chosen)
+                              : a.cluster_max;
+  if (kCluster ? nc > cluster_max : nc <= cluster_max) return;  // the other kernel's
   int nblk = grid_blocks;  // a cluster: all of its blocks
   if (!kCluster) {
     nblk = (nc + kContactsPerBlock - 1) / kContactsPerBlock;
@@ -1700,7 +1708,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve_batch(const SolveArgs* __
   load_args(args + order[blockIdx.x / kBlocks], s_a);
   __syncthreads();
   if (threadIdx.x == 0) {
-    s_a.cluster_max = kBlocks > 1 ? 0x7fffffff : 0;  // this launch's kind
+    s_a.cluster_max = s_a.cluster_alone = kBlocks > 1 ? 0x7fffffff : 0;  // this launch's kind
     s_a.small_max = kSmallContacts;
   }
   __syncthreads();
@@ -2559,7 +2567,7 @@ cudaError_t launch_solve(const SolveArgs& a, int grid_blocks, int cluster_blocks
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k_solve<true>, args);
     if (e != cudaSuccess) return e;
   } else {
-    args.cluster_max = 0;
+    args.cluster_max = args.cluster_alone = 0;
     args.small_max = 0;
   }
   void* params[] = {&args};
