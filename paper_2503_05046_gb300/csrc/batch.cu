@@ -197,16 +197,25 @@ std::vector<int2> build_work(mpm_batch* b) {
 
 // Blocks per scene's contact solve: as asked for, else by how many scenes share
 // the device, each line where the measured times cross (ms per step of four
-// substeps with 1, 2, 4 and 8 blocks; scenes of 2k particles up to the bound):
-//    24 scenes to 64k   4.27  2.65  1.99  1.71
-//    64 scenes to 32k   4.61  3.31  2.69  3.20
-//   128 scenes to 16k   4.04  3.18  2.79  3.59
-//   304 scenes to 8k    4.00  3.53  3.81  5.23
-//   400 scenes to 8k    4.71  4.51  5.00  6.70
+// substeps with 1, 2, 4 and 8 blocks, scenes of 2k particles up to the bound; left
+// the step of touch-down, 20 to 60 iterations per substep in the worst scene, right
+// three steps on):
+//    24 scenes to 64k    23.6  17.1   9.7   8.4     3.46  2.28  1.69  1.38
+//    38 scenes to 48k    39.6  22.1  14.2  11.4     3.54  2.45  1.82  1.61
+//    64 scenes to 32k    70.1  39.2  24.4  26.8     3.62  2.47  1.97  2.21
+//   152 scenes to 16k    61.6  44.3  39.6  63.2     3.15  2.47  2.37  3.12
+//   200 scenes to 12k    55.2  39.7  47.7  83.8     2.88  2.39  2.58  3.52
+//   250 scenes to 8k     44.6  46.7  61.9   107     2.55  2.40  2.74  3.83
+//   304 scenes to 8k     50.8  53.5  72.1   130     2.70  2.67  3.04  4.33
+//   456 scenes to 8k     61.5  73.7   103   189     3.48  3.67  4.33  6.36
+//   800 scenes to 4k     84.6   114   165   348     3.82  4.08  4.76  7.30
+// A device that schedules no cluster of that many blocks takes fewer.
 int solve_blocks_of(const mpm_batch* b) {
   if (b->solve_blocks > 0) return b->solve_blocks;
   const int ns = (int)b->ctx.size(), sms = b->ctx[0]->num_sms;
-  return 4 * ns <= sms ? 8 : ns <= sms ? 4 : ns <= 3 * sms ? 2 : 1;
+  int blocks = 4 * ns <= sms ? 8 : ns <= sms ? 4 : 2 * ns <= 3 * sms ? 2 : 1;
+  while (blocks > 1 && blocks > b->ctx[0]->cluster_blocks_max) blocks /= 2;
+  return blocks;
 }
 
 cudaError_t enqueue(mpm_batch* b, int n_substeps, double dt) {
