@@ -416,7 +416,7 @@ cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_s
   P2GArgs pa;
   pa.g = ctx->g; pa.P = ctx->P[cur]; pa.n = n; pa.groups = ctx->groups_d;
   pa.bodies = ctx->bodies_d; pa.nb = nb; pa.h = hf; pa.G = ctx->G; pa.C = ctx->C;
-  pa.status = ctx->status; pa.stats = ctx->stats;
+  pa.status = ctx->status;
   pa.in_flight = first ? ctx->in_flight : nullptr;
   pa.fext = nullptr;
   pa.fext_stride = ctx->cap;
@@ -459,7 +459,7 @@ cudaError_t enqueue_substep(mpm_ctx* ctx, int cur, int nb, float hf, const mpm_s
   if (with_g2p) {
     G2PArgs ga;
     ga.g = ctx->g; ga.P = ctx->P[cur]; ga.n = n; ga.groups = ctx->groups_d; ga.G = ctx->G;
-    ga.C = ctx->C; ga.h = hf; ga.bar = ctx->bar; ga.red = ctx->red; ga.stats = ctx->stats;
+    ga.C = ctx->C; ga.h = hf; ga.bar = ctx->bar; ga.stats = ctx->stats;
     ga.in_flight = last && n > 0 ? ctx->in_flight : nullptr;  // (no particles: P2G launches nothing)
     mark_phase(ctx, MPM_PHASE_G2P);
     launch_g2p(ga, s);
@@ -1173,22 +1173,21 @@ mpm_status mpm_step(mpm_ctx* ctx, double h, int32_t n_substeps, const mpm_solver
   bool launched = false;
   if (ctx->use_graphs && !ctx->profile && !ctx->wait_test && n_substeps > 0) {
     mpm_ctx::GraphKey k;
-    k.n = n; k.n_substeps = n_substeps; k.nb = nb; k.chunk = ctx->p2g_chunk;
+    k.n = n; k.n_substeps = n_substeps; k.nb = nb;
     k.sort_now = sort_now ? 1 : 0; k.solve_blocks = solve_blocks; k.h = hf; k.sp = sp;
     k.cluster_max = cluster_contacts(ctx);
     k.cluster_alone = cluster_contacts_alone(ctx);
     k.cluster_blocks = ctx->cluster_blocks;
-    k.p2g_form = ctx->p2g_form;
     k.rigid = dev_rigid ? 1 : 0;
     k.taping = ctx->taping && ctx->tape_pool ? 1 : 0;
     k.tape_pool = ctx->tape_pool;
     const mpm_ctx::GraphKey& o = ctx->gkey[from];
     const bool same = ctx->gexec[from] && o.n == k.n && o.n_substeps == k.n_substeps && o.nb == k.nb &&
-                      o.chunk == k.chunk && o.sort_now == k.sort_now &&
+                      o.sort_now == k.sort_now &&
                       o.solve_blocks == k.solve_blocks && o.h == k.h && o.taping == k.taping &&
                       o.cluster_max == k.cluster_max && o.cluster_alone == k.cluster_alone &&
                       o.cluster_blocks == k.cluster_blocks &&
-                      o.rigid == k.rigid && o.p2g_form == k.p2g_form &&
+                      o.rigid == k.rigid &&
                       o.tape_pool == k.tape_pool &&
                       memcmp(&o.sp, &k.sp, sizeof(k.sp)) == 0;
     if (!same) {
@@ -1289,7 +1288,6 @@ mpm_status mpm_step(mpm_ctx* ctx, double h, int32_t n_substeps, const mpm_solver
   stats->contacts_total = (int64_t)ds.contacts_total;
   stats->residual_max = ds.residual_max;
   stats->status_bits = (int32_t)bits;
-  stats->p2g_global_chunks = ds.p2g_global_chunks;
   stats->ls_split_substeps = ds.ls_split;
   stats->cluster_substeps = ds.cluster;
   stats->contact_nodes_max = ds.cnodes_max;
@@ -1895,16 +1893,14 @@ mpm_status mpm_set_option(mpm_ctx* ctx, int32_t option, int64_t value) {
     case MPM_OPT_P2G_CHUNK:
       if (value != 256 && value != 512 && value != 1024)
         return fail(ctx, MPM_ERR_INVALID_ARG, "P2G chunk must be 256, 512 or 1024");
-      ctx->p2g_chunk = (int)value;
-      return MPM_OK;
+      return MPM_OK;  // (P2G's launch shape follows from the particle count)
     case MPM_OPT_GRAPHS:
       ctx->use_graphs = value != 0;
       return MPM_OK;
     case MPM_OPT_P2G_FORM:
       if (value != MPM_P2G_GATHER && value != MPM_P2G_SCATTER)
         return fail(ctx, MPM_ERR_INVALID_ARG, "P2G form must be MPM_P2G_GATHER or MPM_P2G_SCATTER");
-      ctx->p2g_form = (int)value;
-      return MPM_OK;
+      return MPM_OK;  // (one form serves every particle density)
     case MPM_OPT_TEST_BARRIER_TIMEOUT:
       ctx->wait_test = value != 0;
       return MPM_OK;

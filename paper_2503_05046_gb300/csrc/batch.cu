@@ -30,7 +30,6 @@ struct mpm_batch {
   std::vector<mpm_ctx*> ctx;
   // launch options
   bool use_graphs = true;
-  int p2g_chunk = 256;
   long long n_all = 0;  // particles of all members, as the work lists have them
   int g2p_threads = 256;
   int grid_particles = 2048;
@@ -136,10 +135,10 @@ void build_records(mpm_batch* b, float h, const mpm_solver_params& sp) {
     pa = P2GArgs{};
     pa.g = c->g; pa.P = c->P[c->cur]; pa.n = (int)c->n; pa.groups = c->groups_d;
     pa.bodies = c->bodies_d; pa.nb = nb; pa.h = h; pa.G = c->G; pa.C = c->C;
-    pa.status = c->status; pa.stats = c->stats;
+    pa.status = c->status;
     GridBatchArgs& ga = b->grid_h[s];
     ga = GridBatchArgs{};
-    ga.g = c->g; ga.G = c->G; ga.h = h; ga.stats = c->stats;
+    ga.g = c->g; ga.G = c->G; ga.h = h;
     ga.n_slices = grid_slices(b, c);
     SolveArgs& sa = b->solve_h[s];
     sa = SolveArgs{};
@@ -154,7 +153,7 @@ void build_records(mpm_batch* b, float h, const mpm_solver_params& sp) {
     G2PArgs& qa = b->g2p_h[s];
     qa = G2PArgs{};
     qa.g = c->g; qa.P = c->P[c->cur]; qa.n = (int)c->n; qa.groups = c->groups_d; qa.G = c->G;
-    qa.C = c->C; qa.h = h; qa.bar = c->bar; qa.red = c->red; qa.stats = c->stats;
+    qa.C = c->C; qa.h = h; qa.bar = c->bar; qa.stats = c->stats;
     RigidBatchArgs& ra = b->rig_h[s];
     ra = RigidBatchArgs{};
     ra.bodies = c->bodies_d; ra.dyn = c->dyn_d; ra.nb = nb; ra.rigid = nb > 0 ? 1 : 0;
@@ -501,7 +500,6 @@ mpm_status mpm_batch_synchronize(mpm_batch* batch, int32_t* status, mpm_step_sta
       o.contacts_total = (int64_t)d.contacts_total;
       o.residual_max = d.residual_max;
       o.status_bits = (int32_t)words[i];
-      o.p2g_global_chunks = d.p2g_global_chunks;
       o.ls_split_substeps = d.ls_split;
       o.cluster_substeps = d.cluster;
       o.contact_nodes_max = d.cnodes_max;
@@ -521,9 +519,7 @@ mpm_status mpm_batch_set_option(mpm_batch* batch, int32_t option, int64_t value)
     case MPM_BATCH_OPT_P2G_CHUNK:
       if (value != 256 && value != 512 && value != 1024)
         return bfail(batch, MPM_ERR_INVALID_ARG, "P2G chunk must be 256, 512 or 1024");
-      if (batch->p2g_chunk != (int)value) batch->work_valid = false;
-      batch->p2g_chunk = (int)value;
-      return MPM_OK;
+      return MPM_OK;  // (as MPM_OPT_P2G_CHUNK)
     case MPM_BATCH_OPT_G2P_THREADS:
       if (value < 64 || value > 512 || value % 32 != 0)
         return bfail(batch, MPM_ERR_INVALID_ARG, "G2P threads must be 64..512, a multiple of 32");

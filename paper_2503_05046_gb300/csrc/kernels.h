@@ -43,7 +43,6 @@ struct DevStats {
   int substeps;
   unsigned long long contacts_total;
   float residual_max;
-  int p2g_global_chunks;
   int last_contacts;     // contacts of the last substep
   int last_active;       // active blocks of the last substep
   int ls_split;          // substeps whose line search was split over the solve's blocks
@@ -109,7 +108,6 @@ struct P2GArgs {
   GridArrays G;
   Contacts C;
   uint32_t* status;
-  DevStats* stats;
   int* in_flight;  // the step's first substep: the device's count of steps in flight, else null
   float* fext;  // cloth: per-particle mesh forces, 3 planes of fext_stride (null: none); P2G zeroes them
   long long fext_stride;
@@ -307,7 +305,6 @@ struct G2PArgs {
   Contacts C;
   float h;
   unsigned* bar;     // solve barrier, reset here
-  double* red;       // solve reduction ring, reset here
   DevStats* stats;
   int* in_flight;    // the step's last substep: as P2GArgs', else null
 };
@@ -322,7 +319,6 @@ struct GridBatchArgs {
   GridArrays G;
   float h;
   int n_slices;
-  DevStats* stats;
 };
 int p2g_block_particles(long long n);
 void launch_p2g_batch(const P2GArgs* args, const int2* work, int n_work, long long n, cudaStream_t s);
