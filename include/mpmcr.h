@@ -199,8 +199,10 @@ typedef struct {
      blocks, each pass ending in a device-wide reduction (more contacts than
      one block line-searches alone) */
   int32_t ls_split_substeps;
-  /* substeps whose contact solve ran in one thread-block cluster (at most
-     MPM_OPT_CLUSTER_CONTACTS contacts) */
+  /* substeps whose contact solve needed no device-wide barrier: it ran in one
+     thread-block cluster (at most MPM_OPT_CLUSTER_CONTACTS contacts), or in one
+     thread block's shared memory (up to 320 contacts whose nodes fit; counted by
+     mpm_get_one_block_solves alone) */
   int32_t cluster_substeps;
   /* grid nodes in the stencil of at least one contact (the solve's DoFs), in
      one substep */
@@ -550,6 +552,11 @@ enum {
   MPM_PHASE_G2P = 4,        /* grid-to-particle + constitutive update */
   MPM_NUM_PHASES = 5
 };
+
+/* Substeps of the last mpm_step (or of the last mpm_batch_step of the context's
+   batch) whose contact solve ran in one thread block's shared memory: a part of
+   mpm_step_stats.cluster_substeps. Synchronises. */
+mpm_status mpm_get_one_block_solves(mpm_ctx* ctx, int32_t* substeps);
 
 /* Accumulated milliseconds and launch counts per phase since the last reset
    (arrays of MPM_NUM_PHASES; either may be NULL). Synchronises. */

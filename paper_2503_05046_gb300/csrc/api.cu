@@ -1295,6 +1295,15 @@ mpm_status mpm_step(mpm_ctx* ctx, double h, int32_t n_substeps, const mpm_solver
   return st;
 }
 
+mpm_status mpm_get_one_block_solves(mpm_ctx* ctx, int32_t* substeps) {
+  if (!ctx || !substeps) return MPM_ERR_INVALID_ARG;
+  CU(cudaStreamSynchronize(ctx->stream));
+  DevStats ds;
+  CU(cudaMemcpy(&ds, ctx->stats, sizeof(ds), cudaMemcpyDeviceToHost));
+  *substeps = ds.one_block;
+  return MPM_OK;
+}
+
 mpm_status mpm_get_rigid_impulses(mpm_ctx* ctx, double* out, int32_t reset) {
   if (!ctx || (!out && !ctx->bodies.empty())) return MPM_ERR_INVALID_ARG;
   CU(cudaStreamSynchronize(ctx->stream));

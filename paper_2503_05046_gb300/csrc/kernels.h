@@ -46,7 +46,8 @@ struct DevStats {
   int last_contacts;     // contacts of the last substep
   int last_active;       // active blocks of the last substep
   int ls_split;          // substeps whose line search was split over the solve's blocks
-  int cluster;           // substeps solved by one thread-block cluster
+  int cluster;           // substeps solved by one thread-block cluster or one block
+  int one_block;         // of these, the ones solved in one block's shared memory
   int cnodes_max;        // contact nodes (the union of the contacts' stencils) in one substep
   // device time of the contact solve's phases (ns, block 0's view):
   // contact-node list, G, N, line search, impulses

@@ -617,7 +617,7 @@ __device__ __forceinline__ void contact_impulses(const SolveArgs& a, const DevBo
 
 // one thread's record of a finished solve
 __device__ __forceinline__ void solve_stats(const SolveArgs& a, const unsigned long long (&tph)[5],
-                                            int it, int ls_passes, bool split, bool cluster, int ncn,
+                                            int it, int ls_passes, bool split, bool cluster, bool one_block, int ncn,
                                             float resid) {
 #pragma unroll
   for (int k = 0; k < 5; ++k) atomicAdd(&a.stats->solve_ns[k], tph[k]);
@@ -626,6 +626,7 @@ __device__ __forceinline__ void solve_stats(const SolveArgs& a, const unsigned l
   atomicAdd(&a.stats->ls_evals_total, ls_passes);
   if (split) atomicAdd(&a.stats->ls_split, 1);
   if (cluster) atomicAdd(&a.stats->cluster, 1);
+  if (one_block) atomicAdd(&a.stats->one_block, 1);
   atomicMax(&a.stats->cnodes_max, ncn);
   atomicMax(reinterpret_cast<int*>(&a.stats->residual_max), __float_as_int(resid));
 }
@@ -1148,7 +1149,7 @@ __device__ __forceinline__ void small_solve(const SolveArgs& a) {
   lap(4);
   if (tid == 0) {
     clk.finish();
-    solve_stats(a, clk.t, it, ls_passes, false, true, nn, resid);
+    solve_stats(a, clk.t, it, ls_passes, false, true, true, nn, resid);
   }
 }
 
@@ -1668,7 +1669,7 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
   lap(4);
   if (gtid == 0) {
     clk.finish();
-    solve_stats(a, clk.t, it, ls_passes, !local_ls, kCluster, ncn, resid);
+    solve_stats(a, clk.t, it, ls_passes, !local_ls, kCluster, false, ncn, resid);
   }
 }
 

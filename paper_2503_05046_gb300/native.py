@@ -132,6 +132,7 @@ SIGNATURES = {
                      C.POINTER(AdjointParams), C.POINTER(BackwardStats)],
     "mpm_synchronize": [_vp],
     "mpm_set_option": [_vp, C.c_int32, C.c_int64],
+    "mpm_get_one_block_solves": [_vp, _i32p],
     "mpm_get_phase_times": [_vp, _dp, _i64p, C.c_int32],
     "mpm_batch_create": [C.POINTER(_vp), C.c_int32, C.POINTER(_vp)],
     "mpm_batch_step": [_vp, C.c_double, C.c_int32, C.POINTER(SolverParams)],
@@ -454,6 +455,13 @@ def mpm_synchronize(ctx):
 
 def mpm_set_option(ctx, option, value):
     _check(ctx, lib.mpm_set_option(ctx, int(option), int(value)))
+
+
+def mpm_get_one_block_solves(ctx):
+    """Substeps of the last step whose contact solve ran in one thread block."""
+    n = C.c_int32()
+    _check(ctx, lib.mpm_get_one_block_solves(ctx, C.byref(n)))
+    return n.value
 
 
 def mpm_get_phase_times(ctx, reset=False):
