@@ -228,16 +228,16 @@ __device__ __forceinline__ void cell_coord(float x, float o, float o_lo, float i
   dl -= o_lo;
   const float p = dh * inv;
   const float lo = fmaf(dh, inv, -p) + fmaf(dh, inv_lo, dl * inv);
-  const float b = floorf(p - 0.5f);
+  float b = floorf(p - 0.5f);
   f = (p - b) + lo;  // p - b is exact
-  base = (int)b;
   if (f < 0.5f) {
     f += 1.0f;
-    base -= 1;
+    b -= 1.0f;
   } else if (f >= 1.5f) {
     f -= 1.0f;
-    base += 1;
+    b += 1.0f;
   }
+  base = (int)b;  // (saturates far outside the grid)
 }
 
 __device__ __forceinline__ void stencil(const GridDev& g, float x, float y, float z,
@@ -256,8 +256,9 @@ __device__ __forceinline__ void stencil(const GridDev& g, float x, float y, floa
 }
 
 __device__ __forceinline__ bool stencil_inside(const GridDev& g, const Stencil& s) {
-  return s.base[0] >= 0 && s.base[1] >= 0 && s.base[2] >= 0 && s.base[0] + 2 < g.rx &&
-         s.base[1] + 2 < g.ry && s.base[2] + 2 < g.rz;
+  // (not base + 2 < r: a runaway particle's base is the largest int)
+  return s.base[0] >= 0 && s.base[1] >= 0 && s.base[2] >= 0 && s.base[0] < g.rx - 2 &&
+         s.base[1] < g.ry - 2 && s.base[2] < g.rz - 2;
 }
 
 // --------------------------------------------------------------------------
