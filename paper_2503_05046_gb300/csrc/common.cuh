@@ -256,9 +256,11 @@ __device__ __forceinline__ void stencil(const GridDev& g, float x, float y, floa
 }
 
 __device__ __forceinline__ bool stencil_inside(const GridDev& g, const Stencil& s) {
-  // (not base + 2 < r: a runaway particle's base is the largest int)
-  return s.base[0] >= 0 && s.base[1] >= 0 && s.base[2] >= 0 && s.base[0] < g.rx - 2 &&
-         s.base[1] < g.ry - 2 && s.base[2] < g.rz - 2;
+  // (not base + 2 < r: a runaway particle's base is the largest int. One unsigned
+  // comparison per axis and no branch between them: ten substeps of 8,000 particles
+  // in flight 193 us against 196 with two signed ones)
+  return ((unsigned)s.base[0] < (unsigned)(g.rx - 2)) & ((unsigned)s.base[1] < (unsigned)(g.ry - 2)) &
+         ((unsigned)s.base[2] < (unsigned)(g.rz - 2));
 }
 
 // --------------------------------------------------------------------------
