@@ -88,10 +88,15 @@ __device__ __forceinline__ float update_node(const GridDev& g, const GridArrays&
                     k >= g.rz - g.bc;
   float p2 = 0.f;
   if (mp.x > 0.0f) {
+    // p / m + h g with one rounding: the quotient's remainder goes with h g
     const float inv_m = 1.0f / mp.x;
-    vs.x = wall ? 0.0f : mp.y * inv_m + h * g.gx;
-    vs.y = wall ? 0.0f : mp.z * inv_m + h * g.gy;
-    vs.z = wall ? 0.0f : mp.w * inv_m + h * g.gz;
+    auto vstar = [&](float p, float hg) {
+      const float q = p * inv_m;
+      return fabsf(q) < INFINITY ? q + fmaf(fmaf(-q, mp.x, p), inv_m, hg) : q;
+    };
+    vs.x = wall ? 0.0f : vstar(mp.y, h * g.gx);
+    vs.y = wall ? 0.0f : vstar(mp.z, h * g.gy);
+    vs.z = wall ? 0.0f : vstar(mp.w, h * g.gz);
     vs.w = mp.x;
     if (!wall) p2 = mp.x * (vs.x * vs.x + vs.y * vs.y + vs.z * vs.z);
   }

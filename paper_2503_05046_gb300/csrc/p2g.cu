@@ -67,9 +67,11 @@ __device__ __forceinline__ bool box_may_touch(const DevBody& b, float c0, float 
 // pre-reduction that it replaces: 1M elastic particles at 8 per cell 73 -> 51
 // us, 4M in 32 objects 395 -> 231 us, 1M sand at one per cell 126 -> 94 us,
 // 250,000 sand at four per cell 30.5 -> 22.5 us, 8,000 particles 12.0 -> 8.9 us.
-// A node takes more, smaller sums than from a window per block: ten substeps of 1M
-// elastic particles in flight are 1.56e-7 (v) and 1.28e-5 (C) off 64 bits, 1.54e-7
-// and 1.26e-5 with the gather; sand in flight the same with both.
+// A node takes more, smaller sums than from a window per block, which rounds a
+// little more: ten substeps of elastic particles in flight were 1.02 (1M) to 1.07
+// times (36,000 on a sparse grid) as far from 64 bits in v and C. The grid update's
+// single rounding and G2P's differences take off more than that (0.93 to 1.00 of
+// the error with the window and the sums over v_i; sand the same with all).
 //
 // Rounds: a warp that takes three sets gives each walker a set of its own and
 // cuts fewer cells between walkers; with few particles one set per warp spreads
