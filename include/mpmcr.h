@@ -383,7 +383,10 @@ mpm_status mpm_get_contacts(mpm_ctx* ctx, int64_t cap, int64_t* count, int32_t* 
    body of the last step, dL/dv (3) and dL/domega (3) of its spatial velocity
    (through b only: v_r(x) = v + omega x (x - p)) and dL/dmu.
    params may be NULL for eps_r = 1e-5 (stop when the residual's P^-1 norm
-   falls below eps_r times vbar's) and max_iters = 1000.
+   falls below eps_r times vbar's; P is about the nodes' masses, so a vbar that
+   does not shrink with a nearly massless node's mass, as one from a particle's
+   weights does, makes the norm that node's and wants a smaller eps_r) and
+   max_iters = 1000.
    Errors: MPM_ERR_STATE before any mpm_step with n_substeps > 0;
    MPM_ERR_INVALID_ARG for bad arguments or (host ids) an id outside the
    grid, checked before any work; device ids outside the grid are reported
