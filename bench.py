@@ -58,6 +58,12 @@ G2P_BYTES_PER_PARTICLE = 144       # read x, F; write x, v, C, F
 SOLVE_BYTES_PER_CONTACT = 48       # per QN iteration: the contact record
 SOLVE_BYTES_PER_NODE = 60          # per QN iteration and contact node: v, v*, m, g, H, dv
 L2_FLUSH_BYTES = 256 * 1024 * 1024
+# untimed steps after the warm-up, so that the timed ones are always the same
+# part of the motion: the objects have landed and the jaws have closed
+SETTLE_STEPS = 7
+# P2G's line in profiles/traffic.txt, named by its options' default values (which
+# have no effect)
+P2G_TRAFFIC = "p2g_gather_256"
 
 
 def dist_env():
@@ -252,10 +258,8 @@ def measure_workload(native, sc, args, ws, stream_flush=True, tight=True):
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device="cuda")
     for _ in range(args.warmup):
         sim.step(solver=solver, stats=False, check=False)
-    # the P2G form that is faster on this workload, timed on ordinary steps
-    from paper_2503_05046_gb300 import tune
-    (p2g_form, p2g_chunk), form_table = tune.tune_p2g_form(sim, solver, steps=2)
-    sim.step(solver=solver, stats=False, check=False)  # records the step's graph again
+    for _ in range(SETTLE_STEPS):
+        sim.step(solver=solver, stats=False, check=False)
     sim.step(n_substeps=0, solver=solver, check=False)  # drain warm-up status
 
     def timed_steps(k, stats=None):
@@ -333,9 +337,6 @@ def measure_workload(native, sc, args, ws, stream_flush=True, tight=True):
     act_nodes = max(x.active_blocks_max for x in prof_stats) * 64
 
     out = {"value": value, "ms_per_step": ms / args.steps, "steps": args.steps,
-           "p2g_form": {"chosen": ("gather", "scatter")[p2g_form], "particles_per_block": p2g_chunk,
-                        "p2g_us_per_launch": {"%s_%d" % (("gather", "scatter")[f], c): 1e3 * t
-                                              for (f, c), t in form_table}},
            "e2e": {"value": e2e_value, "unit": UNIT, "steps": e2e_steps,
                    "h2d_bytes_per_step": int(nb * C_sizeof_body(native)),
                    "d2h_bytes_per_step": int(12 * n + 48 * nb),
@@ -349,7 +350,6 @@ def measure_workload(native, sc, args, ws, stream_flush=True, tight=True):
                       "residual_max": max(x.residual_max for x in prof_stats),
                       "active_blocks_max": max(x.active_blocks_max for x in prof_stats),
                       "status_bits": functools.reduce(lambda u, x: u | x.status_bits, prof_stats, 0),
-                      "p2g_global_chunks": sum(x.p2g_global_chunks for x in prof_stats),
                       "status_timed": native.STATUS_NAMES[code_timed],
                       "solve_phases_us_per_substep": dict(zip(
                           ("node_list", "gradient_hessian", "node_solve", "line_search", "impulses"),
@@ -388,10 +388,7 @@ def measure_workload(native, sc, args, ws, stream_flush=True, tight=True):
     wl = workload_name(sc)
     out["roofline"] = {"kernel": dom, "bound": "hbm", "achieved": kern[dom]["GBps"], "peak": peak,
                        "peak_kind": peak_kind, "unit": "GB/s", "frac": kern[dom]["GBps"] / peak,
-                       "traffic": profiled_traffic(
-                           dom if dom != "p2g" else "p2g_%s_%d" % (("gather", "scatter")[p2g_form], p2g_chunk),
-                           wl, n),
-                       "form": ("gather", "scatter")[p2g_form] if dom == "p2g" else None,
+                       "traffic": profiled_traffic({"p2g": P2G_TRAFFIC}.get(dom, dom), wl, n),
                        "note": "the streaming kernel with the largest share of the step; the "
                                "contact solve (%.0f%% of the step) is latency-bound, its "
                                "bytes in kernels.solve" % (100.0 * phase_ms["solve"] /
@@ -445,7 +442,7 @@ def run_ours(args):
         "gpu_launches": head["launches_per_step"] * args.steps,
         "roofline": head["roofline"],
     }
-    for key in ("kernels", "phase_ms_per_step", "ms_per_step_profiled", "solver", "tight_solve", "p2g_form"):
+    for key in ("kernels", "phase_ms_per_step", "ms_per_step_profiled", "solver", "tight_solve"):
         if key in head:
             line[key] = head[key]
     if clk:
@@ -522,20 +519,11 @@ def cloth_box_bagging(native, steps=40, warmup=3):
     side included: context, not a like-for-like figure."""
     import torch
     from paper_2503_05046_gb300 import scenes
-    from paper_2503_05046_gb300 import tune
     sc, dyn = scenes.box_bagging()
     solver = native.solver_params(eps_r=5e-2, max_iters=2000)
     N, h = sc["substeps"], sc["h"]
-    # the P2G form, chosen on a copy of the scene so that the measured steps
-    # start from the same state whichever form wins
-    probe = native.Sim(sc)
-    probe.set_dynamics(1, dyn)
-    (form, chunk), _ = tune.tune_p2g_form(probe, solver, steps=2)
-    probe.close()
     sim = native.Sim(sc)
     sim.set_dynamics(1, dyn)
-    native.mpm_set_option(sim.ctx, native.OPT_P2G_FORM, form)
-    native.mpm_set_option(sim.ctx, native.OPT_P2G_CHUNK, chunk)
     for _ in range(warmup):
         sim.step(solver=solver, check=False)
     st0 = sim.get_particles()
@@ -566,7 +554,6 @@ def cloth_box_bagging(native, steps=40, warmup=3):
            "us_per_substep": 1e3 * ms / N, "particle_substeps_per_s": n * N / (ms * 1e-3),
            "real_time_rate": N * h / (ms * 1e-3), "eps_r": 5e-2, "contacts_max": contacts,
            "iters_per_substep": iters / max(subs, 1), "steps_not_converged": failed,
-           "p2g_form": ("gather", "scatter")[form],
            "box_drop_m": float(b0[1]["p"][2] - box_end["p"][2]),
            "paper": {"ms_per_step": 45.3, "particles": 2582, "substeps_per_step": 10,
                      "hardware": "RTX 4090, rigid and robot side included"}}
@@ -579,12 +566,12 @@ def batched_throughput(native, n_scenes=256, steps=3, warmup=2, ws=1, rank=0):
     sand, a gripper jaw and the ground) advanced three ways, each timed by the
     host clock around `steps` steps of every scene, synchronised on both sides:
     - `value`: one batch (mpm_batch_*): a substep of all scenes is one P2G, one
-      compaction, one grid-update, one contact-solve and one G2P launch over
-      (scene, block) work items, the time step one CUDA graph; launch options
-      picked by tune.tune_batch_launch;
+      grid-update, two contact-solve (few contacts, and more) and one G2P launch
+      over (scene, block) work items, the time step one CUDA graph; launch
+      options picked by tune.tune_batch_launch;
     - `concurrent_value`: one context per scene, each on its own stream
       replaying its own step graph, enqueued one after another without
-      waiting, SM cap of the solve and P2G block size by tune.tune_batch;
+      waiting, SM cap of the solve by tune.tune_batch;
     - `loop_value`: the single-scene path looped (one scene at a time, every
       step waited for, default options).
     On several GPUs the scenes are split round robin over the ranks (they
@@ -617,12 +604,11 @@ def batched_throughput(native, n_scenes=256, steps=3, warmup=2, ws=1, rank=0):
 
     # (2) contexts side by side, (3) the loop
     sims = [native.Sim(sc, max_contacts=2 * scenes.n_particles(sc)) for sc in scs]
-    (solve_cap, chunk), table = tune.tune_batch(sims, scs, solver)
+    (solve_cap, _), table = tune.tune_batch(sims, scs, solver)
 
-    def run(cap, wait_each, p2g_chunk=256):
+    def run(cap, wait_each):
         for sim in sims:
             native.mpm_set_option(sim.ctx, native.OPT_SOLVE_BLOCKS, cap)
-            native.mpm_set_option(sim.ctx, native.OPT_P2G_CHUNK, p2g_chunk)
         for _ in range(warmup):
             for sim, sc in zip(sims, scs):
                 native.mpm_step(sim.ctx, sc["h"], sc["substeps"], solver, want_stats=False)
@@ -639,7 +625,7 @@ def batched_throughput(native, n_scenes=256, steps=3, warmup=2, ws=1, rank=0):
         torch.cuda.synchronize()
         return max_over_ranks(time.perf_counter() - t0, ws)
 
-    t_conc = run(solve_cap, False, chunk)
+    t_conc = run(solve_cap, False)
     codes = [native.mpm_synchronize(sim.ctx) for sim in sims]
     t_loop = run(0, True)
     for sim in sims:
@@ -647,7 +633,7 @@ def batched_throughput(native, n_scenes=256, steps=3, warmup=2, ws=1, rank=0):
     v_persist = n_scenes * steps / t_persist
     v_conc = n_scenes * steps / t_conc
     v_loop = n_scenes * steps / t_loop
-    names = {native.BATCH_OPT_P2G_CHUNK: "p2g_chunk", native.BATCH_OPT_G2P_THREADS: "g2p_threads",
+    names = {native.BATCH_OPT_G2P_THREADS: "g2p_threads",
              native.BATCH_OPT_GRID_PARTICLES: "grid_particles_per_block",
              native.BATCH_OPT_SOLVE_BLOCKS: "solve_blocks_per_scene"}
     return {"scenes": n_scenes, "particles": n_total, "steps": steps, "substeps_per_step": N,
@@ -658,15 +644,14 @@ def batched_throughput(native, n_scenes=256, steps=3, warmup=2, ws=1, rank=0):
             "launches_per_step": 2 + 5 * N,
             "concurrent_value": v_conc, "loop_value": v_loop,
             "speedup_vs_concurrent": v_persist / v_conc, "speedup_vs_loop": v_persist / v_loop,
-            "tuned": {names[k]: v for k, v in best.items()},
-            "tuning_s_per_2_steps": [[{names[k]: v for k, v in c.items()}, round(t, 4)]
+            "tuned": {names[k]: v for k, v in best.items() if k in names},
+            "tuning_s_per_2_steps": [[{names[k]: v for k, v in c.items() if k in names}, round(t, 4)]
                                      for c, t in table_b],
             "contacts_per_scene": [int(min(contacts_b)), int(max(contacts_b))],
             "status": "ok" if code_b == 0 else
                       "%d scenes reported %s" % (int(np.sum(codes_b != 0)), sorted(set(codes_b.tolist()))),
-            "concurrent_tuned": {"solve_cap": solve_cap, "p2g_chunk": chunk,
-                                 "candidates_s_per_2_steps": [[c, k, round(t, 4)]
-                                                              for c, k, t in table]},
+            "concurrent_tuned": {"solve_cap": solve_cap,
+                                 "candidates_s_per_2_steps": [[c, round(t, 4)] for c, _, t in table]},
             "status_concurrent": "ok" if all(c == 0 for c in codes) else
                                  "%d scenes reported %s" % (sum(c != 0 for c in codes), sorted(set(codes))),
             "timing": "host clock around the enqueue loop, synchronised on both sides"}
