@@ -626,7 +626,7 @@ mpm_status mpm_batch_synchronize(mpm_batch* batch, int32_t* status, mpm_step_sta
    MPM_BATCH_OPT_SOLVE_BLOCKS: thread blocks per scene's contact solve, 1, 2, 4
      or 8 (more than one form a thread-block cluster per scene); unset, the
      batch picks by its scene count (on GB300 8 up to 38 scenes, 4 up to 152, 2
-     up to 228). The solves start largest scene (by particle count) first. */
+     up to 228, or 456 if the largest has 12,000 particles or more). The solves start largest scene (by particle count) first. */
 enum {
   MPM_BATCH_OPT_GRAPHS = 1,
   MPM_BATCH_OPT_P2G_CHUNK = 2,

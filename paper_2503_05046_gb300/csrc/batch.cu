@@ -195,24 +195,31 @@ std::vector<int2> build_work(mpm_batch* b) {
 }
 
 // Blocks per scene's contact solve: as asked for, else by how many scenes share
-// the device, each line where the measured times cross (ms per step of four
-// substeps with 1, 2, 4 and 8 blocks, scenes of 2k particles up to the bound; left
-// the step of touch-down, 20 to 60 iterations per substep in the worst scene, right
-// three steps on):
-//    24 scenes to 64k    23.6  17.1   9.7   8.4     3.46  2.28  1.69  1.38
-//    38 scenes to 48k    39.6  22.1  14.2  11.4     3.54  2.45  1.82  1.61
-//    64 scenes to 32k    70.1  39.2  24.4  26.8     3.62  2.47  1.97  2.21
-//   152 scenes to 16k    61.6  44.3  39.6  63.2     3.15  2.47  2.37  3.12
-//   200 scenes to 12k    55.2  39.7  47.7  83.8     2.88  2.39  2.58  3.52
-//   250 scenes to 8k     44.6  46.7  61.9   107     2.55  2.40  2.74  3.83
-//   304 scenes to 8k     50.8  53.5  72.1   130     2.70  2.67  3.04  4.33
-//   456 scenes to 8k     61.5  73.7   103   189     3.48  3.67  4.33  6.36
-//   800 scenes to 4k     84.6   114   165   348     3.82  4.08  4.76  7.30
-// A device that schedules no cluster of that many blocks takes fewer.
+// the device and how large the largest is, each line where the measured times cross
+// (ms per step of four substeps with 1, 2, 4 and 8 blocks, scenes of 2k particles up
+// to the bound; left the step of touch-down, 20 to 60 iterations per substep in the
+// worst scene, right three steps on):
+//    38 scenes to 64k    42.7  25.3  20.3  18.5     4.11  2.76  2.21  1.93
+//    64 scenes to 16k    55.1  39.1  26.1  33.7     2.57  1.94  1.59  1.82
+//   152 scenes to 16k    60.8  42.8  38.9  63.1     3.20  2.57  2.52  3.36
+//   152 scenes to 64k    57.9  46.8  36.8  45.0     6.80  5.19  4.94  5.83
+//   200 scenes to 8k     41.0  39.4  48.9  85.4     2.37  2.13  2.35  3.20
+//   256 scenes to 8k     42.3  46.9  63.3   111     2.76  2.56  2.85  4.06
+//   456 scenes to 8k     60.0  73.0   100   189     3.55  3.77  4.42  6.63
+//   256 scenes to 64k    82.5  62.9  54.0  73.6     8.66  7.63  7.94  9.65
+//   340 scenes to 16k    65.2  55.7  68.6   122     4.25  4.12  4.63  6.48
+//   456 scenes to 64k     101  84.2  79.5   123    12.82 12.67 13.50 16.70
+//   700 scenes to 32k     106   104   130   219    11.30 11.78 13.28 17.94
+// Scenes of a few thousand particles have too few contacts for a second block once
+// there are more scenes than 1.5 per SM. A device that schedules no cluster of that
+// many blocks takes fewer.
 int solve_blocks_of(const mpm_batch* b) {
   if (b->solve_blocks > 0) return b->solve_blocks;
   const int ns = (int)b->ctx.size(), sms = b->ctx[0]->num_sms;
-  int blocks = 4 * ns <= sms ? 8 : ns <= sms ? 4 : 2 * ns <= 3 * sms ? 2 : 1;
+  int64_t largest = 0;
+  for (const mpm_ctx* c : b->ctx) largest = c->n > largest ? c->n : largest;
+  const int two = largest >= 12000 ? 3 * sms : 3 * sms / 2;
+  int blocks = 4 * ns <= sms ? 8 : ns <= sms ? 4 : ns <= two ? 2 : 1;
   while (blocks > 1 && blocks > b->ctx[0]->cluster_blocks_max) blocks /= 2;
   return blocks;
 }
