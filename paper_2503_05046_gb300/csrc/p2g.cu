@@ -58,11 +58,12 @@ __device__ __forceinline__ bool box_may_touch(const DevBody& b, float c0, float 
 // records in place: one exposed memory latency per warp instead of two per 32
 // particles (long-scoreboard stalls 2.6 -> 0.9 cycles per issued instruction).
 //
-// Bound by instruction issue (about 1,000 instructions per 32 particles at 8
-// per cell, 60% of the issue slots while warps are resident) and, near one
-// particle per cell, by the walkers' cell changes and the reductions (270-290 G
-// red.v4/s measured on GB300, 0.9 per clock and SM: why columns shared by
-// cells adjacent in x are kept). Measured per launch, against the better of
+// Bound by shared-memory traffic and instruction issue together (1M elastic
+// particles at 8 per cell: the L1's data path 81% busy, 66% of the issue slots,
+// 1,084 instructions per 32 particles) and, near one particle per cell, by the
+// walkers' cell changes and the reductions too (1M sand: 1,779 instructions, 60%,
+// L2 42%; 270-290 G red.v4/s measured on GB300, 0.9 per clock and SM: why columns
+// shared by cells adjacent in x are kept). Measured per launch, against the better of
 // the lane-per-node gather into a shared window and the scatter with a shuffle
 // pre-reduction that it replaces: 1M elastic particles at 8 per cell 73 -> 51
 // us, 4M in 32 objects 395 -> 231 us, 1M sand at one per cell 126 -> 94 us,
@@ -75,15 +76,17 @@ __device__ __forceinline__ bool box_may_touch(const DevBody& b, float c0, float 
 //
 // Rounds: a warp that takes three sets gives each walker a set of its own and
 // cuts fewer cells between walkers; with few particles one set per warp spreads
-// the work over more SMs and shortens each warp's chain (79,000 particles: 12.3
-// against 16.1 us with three; 250,000: 34.9 against 32.6; 1M: 83 against 60).
-// The line lies between.
+// the work over more SMs and shortens each warp's chain. us per launch with one
+// and with three sets: elastic at 8 per cell 79,507 13.3 and 16.4, 125,000 13.7 and
+// 14.8, 157,464 14.6 and 14.1, 250,047 24.7 and 23.0, 1M 59.5 and 51.6; sand at 4 per
+// cell 160,000 18.2 and 20.7, 250,000 22.4 and 22.7; at one per cell 250,000 27.1 and
+// 29.7, 1M 79.6 and 78.4. The line is where the denser one crosses.
 constexpr int kWalkOneRound = 160000;  // fewer particles than this: one set per warp
 constexpr int kWalkThreads = 32;  // a warp per block: blocks spread evenly, and nothing is shared
 constexpr int kRawPlanes = 21;  // x, v, C, tau as copied from the particle planes
 
 // One set of 32 staged particles. It arrives as raw planes and is turned into
-// records in place. 712 words: the walkers' sets start 8 banks apart.
+// records in place. 728 words: the walkers' sets start 24 banks apart.
 struct __align__(16) WalkSet {
   union {
     struct {

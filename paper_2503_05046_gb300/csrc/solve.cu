@@ -1474,8 +1474,8 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, int block, int gr
     float2* slot = next_slot();
     {
       float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // G2, P2 - P*2, J2, A, B
-      // (a node's loads go out while the one before it is worked on: with the
-      // list entry, the node and the step one after the other, a round of a
+      // (a node's loads go out together, and the next list entry with them: with
+      // the list entry, the node and the step one after the other, a round of a
       // thread took 6.5 us)
       struct NodeIn {
         float4 vs, v, vl, d, c0, c1;
